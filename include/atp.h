@@ -76,7 +76,8 @@ enum {
 enum {
     ATP_OPT_COST_FP64 = 1,    /* accumulate the running cost in FP64 (default 0: FP32) */
     ATP_OPT_LANES = 2,        /* threads per candidate in atp_plan / atp_rollout: 0 chooses
-                                 by batch size (default), 1, 2 or 4 forces it */
+                                 by batch size (default), 1, 2 or 4 (eight in a small
+                                 plan) forces it */
     ATP_OPT_STAGE_TERRAIN = 3 /* side in nodes (2..120) of a texel window staged in shared
                                  memory by atp_plan / atp_rollout; 0 (default) off */
 };
@@ -173,10 +174,11 @@ size_t atp_terrain_bytes(int nx, int ny, int format);
  * ATP_OPT_COST_FP64 (value 0 or 1) accumulates each candidate's running cost
  * (time, control effort and the soft ESM and costmap constraints, Sec. IV-C)
  * in FP64 instead of FP32; ATP_OPT_LANES (0, 1, 2 or 4) sets the threads per
- * candidate of atp_plan and atp_rollout (two split the axles and four the
- * wheels: lower latency for small batches; one: more throughput once a batch
- * fills the GPU).  One, two and four lanes give the same bits: every layout
- * forms the axle sums and the force and moment totals in one order.
+ * candidate of atp_plan and atp_rollout (one: more throughput once a batch
+ * fills the GPU; two and four, in two warps that share the candidates' Euler
+ * steps: lower latency for smaller batches; four means eight in plans of up to
+ * 4864 candidates).  Every layout gives the same bits: all form the axle sums
+ * and the force and moment totals in one order.
  * ATP_OPT_STAGE_TERRAIN (0, or a side W from 2 to 120 nodes) stages a window
  * of the texels in shared memory (Sec. IV-D's cached terrain lookups): each
  * CTA of 512 threads first copies min(W, nx) x min(W, ny) texels (16 B each,
@@ -272,10 +274,8 @@ typedef struct {
  * Each plan's results are bit-identical to a single atp_plan of the same
  * request, alone or in any mix, since every layout gives the same bits.  The
  * batch chooses each plan's threads per candidate for the batch as a whole:
- * ATP_OPT_LANES if set; else one, raised in request order to the four (or
- * two) lanes a plan of its size would run alone while the batch's threads
- * stay within what a two-lane plan alone may use (2 x 28672), else to two if
- * those fit.  The
+ * ATP_OPT_LANES if set; else the count (one, two, four or eight, the same for
+ * the whole batch) with the smallest estimate of the batch's time.  The
  * context's scratch grows to the sum of the plans' needs; atp_reserve(ctx,
  * sum of N, max H) pre-sizes it for any batch within those totals.
  * Validation failures name the offending request in atp_last_error. */

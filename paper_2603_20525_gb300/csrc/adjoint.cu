@@ -86,17 +86,14 @@ __device__ __forceinline__ Lane lane_of(const Veh &V, int q, unsigned mask)
     return l;
 }
 
-// a lookup axis: cell, weight and whether the query was clamped
-__device__ __forceinline__ int axis_c(int ic, float fc, float o, float inv_cell, int n, float &a, bool &clamped)
+// a lookup axis: cell (magic form), weight and whether the query was clamped
+// (the last node itself counts: the weight there is 1 whatever moves the query)
+__device__ __forceinline__ float axis_c(const Cell &c, float o, float inv_cell, float &a, bool &clamped)
 {
-    const float u = fmaf(o, inv_cell, fc);
-    const float fl = floorf(u);
-    const int i = ic + (int)fmaxf(fminf(fl, 4194304.f), -4194304.f);
-    const float w = u - fl;
-    const bool below = i < 0, above = i >= n - 1;
-    clamped = below || above;
-    a = below ? 0.f : (above ? 1.f : w);
-    return below ? 0 : (above ? n - 2 : i);
+    const float u = fmaf(o, inv_cell, c.fc);
+    bool off = false;
+    clamped = !(u >= c.lo && u < c.hi);
+    return axis(c, u, a, off);
 }
 
 // every intermediate of one wheel that its adjoint needs
@@ -108,8 +105,8 @@ struct WF {
     float tx, ty, tz, itz, Q, chi, A, Bv, N, chid, Fk, Fb0, Fz, alpha, Ca, T, Fy;
 };
 
-__device__ __forceinline__ void wheel_fwd(const Veh &V, const Terrain &T, const float R[9], int icx, float fcx,
-                                          int icy, float fcy, float z, float zl, float vx, float vy, float vz,
+__device__ __forceinline__ void wheel_fwd(const Veh &V, const Terrain &T, const float R[9], const Cell &cx,
+                                          const Cell &cy, unsigned base, float z, float zl, float vx, float vy, float vz,
                                           float wx, float wy, float wz, float rx, float ry, float k, float b,
                                           float Fs, float di, WF &w)
 {
@@ -119,13 +116,14 @@ __device__ __forceinline__ void wheel_fwd(const Veh &V, const Terrain &T, const 
     w.vix = fmaf(-wz, ry, fmaf(-wy, V.hR, vx));
     w.viy = fmaf(wx, V.hR, fmaf(wz, rx, vy));
     w.viz = fmaf(-wy, rx, fmaf(wx, ry, vz));
-    const int i = axis_c(icx, fcx, w.ox, T.inv_cell, T.nx, w.a, w.cx);
-    const int j = axis_c(icy, fcy, w.oy, T.inv_cell, T.ny, w.b, w.cy);
-    const float4 *r0 = T.tex + (size_t)j * T.nx + i;
+    const float tx = axis_c(cx, w.ox, T.inv_cell, w.a, w.cx);
+    const float ty = axis_c(cy, w.oy, T.inv_cell, w.b, w.cy);
+    const unsigned o = texel_index(base, tx, ty, T.nx);
+    const float4 *r0 = T.tex + o, *r1 = T.tex + (size_t)(o + (unsigned)T.nx);
     w.t00 = __ldg(r0);
     w.t10 = __ldg(r0 + 1);
-    w.t01 = __ldg(r0 + T.nx);
-    w.t11 = __ldg(r0 + T.nx + 1);
+    w.t01 = __ldg(r1);
+    w.t11 = __ldg(r1 + 1);
     w.t = lerp4(w.t00, w.t10, w.t01, w.t11, w.a, w.b, T.has_cm != 0);
     w.tx = fmaf(-R[3], w.t.z, fmaf(-R[0], w.t.y, R[6]));
     w.ty = fmaf(-R[4], w.t.z, fmaf(-R[1], w.t.y, R[7]));
@@ -293,13 +291,11 @@ __device__ __forceinline__ StepOut step_fwd(const GradParams &p, St &s, float dd
     R[6] = -sth;
     R[7] = cth * sph;
     R[8] = cph * cth;
-    int icx, icy;
-    float fcx, fcy;
-    cell_split(s.x, s.xl, T.inv_cell, icx, fcx);
-    cell_split(s.y, s.yl, T.inv_cell, icy, fcy);
+    const Cell cx = cell_of<false>(s.x, s.xl, T.inv_cell, T.nx), cy = cell_of<false>(s.y, s.yl, T.inv_cell, T.ny);
+    const unsigned base = texel_base(cx, cy, T.nx);
     const float gBx = -V.g * R[6], gBy = -V.g * R[7], gBz = -V.g * R[8];
     WF w;
-    wheel_fwd(V, T, R, icx, fcx, icy, fcy, s.z, s.zl, s.vx, s.vy, s.vz, s.wx, s.wy, s.wz, ln.rx, ln.ry, ln.k,
+    wheel_fwd(V, T, R, cx, cy, base, s.z, s.zl, s.vx, s.vy, s.vz, s.wx, s.wy, s.wz, ln.rx, ln.ry, ln.k,
               ln.b, ln.Fs, ln.front ? s.d : 0.f, w);
     const float fy = ln.front ? w.Fy * cd : w.Fy;
     const float FyB = qsum(fy, ln.mask);
@@ -371,13 +367,11 @@ __device__ void step_adj(const GradParams &p, const St &s, float dd, float ax, f
     R[6] = -sth;
     R[7] = cth * sph;
     R[8] = cph * cth;
-    int icx, icy;
-    float fcx, fcy;
-    cell_split(s.x, s.xl, T.inv_cell, icx, fcx);
-    cell_split(s.y, s.yl, T.inv_cell, icy, fcy);
+    const Cell cx = cell_of<false>(s.x, s.xl, T.inv_cell, T.nx), cy = cell_of<false>(s.y, s.yl, T.inv_cell, T.ny);
+    const unsigned base = texel_base(cx, cy, T.nx);
     const float vx = s.vx, vy = s.vy, vz = s.vz, wx = s.wx, wy = s.wy, wz = s.wz;
     WF w;
-    wheel_fwd(V, T, R, icx, fcx, icy, fcy, s.z, s.zl, vx, vy, vz, wx, wy, wz, ln.rx, ln.ry, ln.k, ln.b, ln.Fs,
+    wheel_fwd(V, T, R, cx, cy, base, s.z, s.zl, vx, vy, vz, wx, wy, wz, ln.rx, ln.ry, ln.k, ln.b, ln.Fs,
               ln.front ? s.d : 0.f, w);
     const float soft = fmaxf(fmaf(-U, Cc.inv_eps, 1.f), 0.f);
     const float ic = rcp(cth);

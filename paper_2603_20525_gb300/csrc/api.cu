@@ -321,6 +321,42 @@ cudaError_t launch_plan_for(const atp_ctx *ctx, atp::PlanParams &p, const atp_te
     return atp::launch_plan_staged(p, reduce, stream);
 }
 
+// The layout of a batch's plans and the order of their CTAs.  A batch takes at
+// least its slowest plan's Euler steps times the latency of the layout (times
+// the waves of a plan that alone overfills the 912 CTAs resident on 152 SMs),
+// and at least the SMs' time for all its candidates; a layout of more threads
+// shortens the first and costs more of the second.  The layout with the
+// smallest cube root of the two bounds' cubes wins: within 10 % of the measured
+// time on ten serving batches of 1024 to 93184 candidates.  One layout for the
+// whole batch: mixes of layouts were measured slower than either alone (seven
+// plans of 4096: 1.07 ms mixed, 0.74 ms on two threads, 0.91 ms on one; the
+// SMs then alternate between the layouts' loops).  The CTAs go in the order
+// of the plans' Euler steps, the longest first.
+int choose_layout(const atp_plan_request *q, const int *ns, int n)
+{
+    // cycles per Euler step with the GPU nearly idle, and SM cycles per
+    // candidate and Euler step with it full, from a sweep on a GB300
+    constexpr int kL[4] = {atp::kLayoutOne, atp::kLayoutDuo1, atp::kLayoutDuo2, atp::kLayoutDuo4};
+    constexpr double kLatency[4] = {1744., 1273., 1000., 818.}, kBusy[4] = {9.0, 10.3, 12.9, 19.5};
+    constexpr double kSms = 152., kWave = 6 * kSms;
+    double best = INFINITY;
+    int layout = atp::kLayoutOne;
+    for (int l = 0; l < 4; ++l) {
+        double slowest = 0., busy = 0.;
+        for (int r = 0; r < n; ++r) {
+            const double steps = (double)q[r].H * ns[r];
+            slowest = std::max(slowest, steps * kLatency[l] * std::ceil((double)atp::layout_ctas(kL[l], q[r].N) / kWave));
+            busy += steps * q[r].N * (kBusy[l] / kSms);
+        }
+        const double est = slowest * slowest * slowest + busy * busy * busy;
+        if (est < best) {
+            best = est;
+            layout = kL[l];
+        }
+    }
+    return layout;
+}
+
 }  // namespace
 
 extern "C" {
@@ -543,8 +579,8 @@ extern "C" int atp_plan_batch(atp_ctx *ctx, const atp_plan_request *reqs, int n_
     if (!reqs || n_req < 1 || n_req > atp::kMaxBatch)
         return fail(ctx, ATP_ERR_INVALID, "need 1 <= n_req <= %d requests", atp::kMaxBatch);
     size_t need = 0;
-    long long ctas = 0, threads = 0;
-    int ns[atp::kMaxBatch], lanes[atp::kMaxBatch];
+    long long ctas = 0;
+    int ns[atp::kMaxBatch], layout[atp::kMaxBatch], order[atp::kMaxBatch];
     for (int r = 0; r < n_req; ++r) {
         const atp_plan_request &q = reqs[r];
         int rc = common_checks(ctx, q.veh, q.cost, q.terrain, q.x0 ? &q.x0->x : nullptr, 13, q.x0_dev,
@@ -558,33 +594,16 @@ extern "C" int atp_plan_batch(atp_ctx *ctx, const atp_plan_request *reqs, int n_
         if (!q.out_dev) return fail(ctx, ATP_ERR_INVALID, "request %d: out_dev is NULL", r);
         if (q.N > (1 << 29)) return fail(ctx, ATP_ERR_UNSUPPORTED, "request %d: N too large for a batch", r);
         need += region_layout((size_t)q.N, (size_t)q.H, q.best_margin_dev != nullptr).total;
-        lanes[r] = ctx->lanes ? ctx->lanes : 1;
-        threads += (long long)q.N * lanes[r];
     }
-    // Several lanes per candidate pay only while the GPU is mostly empty, and
-    // every layout gives the same bits, so the batch chooses each plan's
-    // lanes for the batch as a whole (unless ATP_OPT_LANES forces them):
-    // every plan starts at one lane, and in request order a plan that would
-    // run four (or two) lanes alone gets them while the batch's threads stay
-    // within what a two-lane plan alone may use, else two if those fit.
-    // Measured on the GB300 on the 32-vehicle serving mix: at 80 requests/s
-    // per vehicle p99 fell from 55 to 32 ms, unchanged at 20 to 40.
-    if (!ctx->lanes) {
-        const long long budget = 2LL * atp::kLanes2MaxN;
-        for (int r = 0; r < n_req; ++r) {
-            const long long N = reqs[r].N;
-            const int alone = atp::plan_lanes(0, reqs[r].N);
-            if (alone == 4 && threads + 3 * N <= budget) {
-                lanes[r] = 4;
-                threads += 3 * N;
-            } else if (alone >= 2 && threads + N <= budget) {
-                lanes[r] = 2;
-                threads += N;
-            }
-        }
+    const int auto_layout = ctx->lanes ? 0 : choose_layout(reqs, ns, n_req);
+    for (int r = 0; r < n_req; ++r) {
+        layout[r] = ctx->lanes ? atp::plan_layout(ctx->lanes, reqs[r].N) : auto_layout;
+        order[r] = r;
     }
-    for (int r = 0; r < n_req; ++r)
-        ctas += ((long long)reqs[r].N * lanes[r] + atp::kPlanBlock - 1) / atp::kPlanBlock;
+    std::stable_sort(order, order + n_req, [&](int a, int b) {
+        return (long long)reqs[a].H * ns[a] > (long long)reqs[b].H * ns[b];
+    });
+    for (int r = 0; r < n_req; ++r) ctas += atp::layout_ctas(layout[r], reqs[r].N);
     if (ctas > 0x7fffffffLL) return fail(ctx, ATP_ERR_UNSUPPORTED, "batch too large");
     DeviceGuard g(ctx->device);
     if (g.err != cudaSuccess) return cuda_fail(ctx, g.err, "set device");
@@ -595,13 +614,13 @@ extern "C" int atp_plan_batch(atp_ctx *ctx, const atp_plan_request *reqs, int n_
     b.cta_begin[0] = 0;
     char *region = (char *)ctx->scratch + kHeaderBytes;
     for (int r = 0; r < n_req; ++r) {
-        const atp_plan_request &q = reqs[r];
+        const atp_plan_request &q = reqs[order[r]];
         const bool steps = q.best_margin_dev != nullptr;
         const RegionLayout L = region_layout((size_t)q.N, (size_t)q.H, steps);
         atp::PlanParams &p = b.req[r];
         std::memset(&p, 0, sizeof p);
         derive(*q.veh, *q.cost, *q.terrain, p);
-        fill_problem(p, q.x0, q.x0_dev, q.ctrl_dev, q.N, q.H, q.dt, ns[r]);
+        fill_problem(p, q.x0, q.x0_dev, q.ctrl_dev, q.N, q.H, q.dt, ns[order[r]]);
         p.cost = q.cand_cost_dev ? q.cand_cost_dev : (float *)(region + L.cost);
         p.margin = q.cand_margin_dev ? q.cand_margin_dev : (float *)(region + L.margin);
         p.flags = q.cand_flags_dev ? q.cand_flags_dev : (uint8_t *)(region + L.flags);
@@ -613,9 +632,9 @@ extern "C" int atp_plan_batch(atp_ctx *ctx, const atp_plan_request *reqs, int n_
         p.best_margin = q.best_margin_dev;
         p.scratch = (atp::Scratch *)ctx->scratch + r;
         p.acc64 = ctx->acc64;
-        p.lanes = lanes[r];
+        p.lanes = layout[order[r]];
         region += L.total;
-        b.cta_begin[r + 1] = b.cta_begin[r] + (int)(((long long)q.N * p.lanes + atp::kPlanBlock - 1) / atp::kPlanBlock);
+        b.cta_begin[r + 1] = b.cta_begin[r] + (int)atp::layout_ctas(p.lanes, q.N);
     }
     cudaError_t e = atp::launch_plan_batch(b, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "batch launch");

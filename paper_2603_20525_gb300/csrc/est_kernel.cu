@@ -22,16 +22,16 @@ namespace atp {
 
 namespace {
 
-// Costmap value at the point (cell icx + fcx + ox / cell, ...): bilinear over
-// the texels' cost channel; sets `off` for a query outside the map.
+// Bilinear lookup at (ox, oy) metres from the CoM; sets `off` for a query
+// outside the map.
 template <int TEX>
-__device__ __forceinline__ float cost_at(const Terrain &T, int icx, float fcx, int icy, float fcy, float ox,
+__device__ __forceinline__ float4 lookup(const Terrain &T, const Cell &cx, const Cell &cy, unsigned base, float ox,
                                          float oy, bool &off)
 {
     float a, b;
-    const int i = axis(icx, fcx, ox, T.inv_cell, T.nx, a, off);
-    const int j = axis(icy, fcy, oy, T.inv_cell, T.ny, b, off);
-    return bilerp<TEX>(T, i, j, a, b).w;
+    const float tx = axis(cx, fmaf(ox, T.inv_cell, cx.fc), a, off);
+    const float ty = axis(cy, fmaf(oy, T.inv_cell, cy.fc), b, off);
+    return bilerp<TEX>(T, cx, cy, base, tx, ty, a, b);
 }
 
 __device__ __forceinline__ float tire(const Veh &V, float Fz, float alpha)
@@ -89,13 +89,10 @@ __device__ __forceinline__ void est_one(const PlanParams &p, int j, float &J, fl
                 continue;
             }
             // terrain under the CoM and its unit normal (reading Q1)
-            int icx, icy;
-            float fcx, fcy, a, b;
-            cell_split(x, xl, T.inv_cell, icx, fcx);
-            cell_split(y, yl, T.inv_cell, icy, fcy);
-            const int ti = axis(icx, fcx, 0.f, T.inv_cell, T.nx, a, off);
-            const int tj = axis(icy, fcy, 0.f, T.inv_cell, T.ny, b, off);
-            const float4 t = bilerp<TEX>(T, ti, tj, a, b);
+            const Cell cx = cell_of(x, xl, T.inv_cell, T.nx), cy = cell_of(y, yl, T.inv_cell, T.ny);
+            const unsigned base = texel_base(cx, cy, T.nx);
+            off = off || off_com(cx, cy);
+            const float4 t = lookup<TEX>(T, cx, cy, base, 0.f, 0.f, off);
             const float rn = rsq(fmaf(t.y, t.y, fmaf(t.z, t.z, 1.f)));
             const float tx = -t.y * rn, ty = -t.z * rn, tz = rn;
             // 1-2-3 angles of the plane: sin(theta) = tau_x, cos(theta) =
@@ -140,10 +137,10 @@ __device__ __forceinline__ void est_one(const PlanParams &p, int j, float &J, fl
                 const float ofx = fmaf(R02, -V.hR, R00 * V.Lf), ofy = fmaf(R12, -V.hR, R10 * V.Lf);
                 const float orx = fmaf(R02, -V.hR, -R00 * V.Lr), ory = fmaf(R12, -V.hR, -R10 * V.Lr);
                 const float lx = R01 * V.he, ly = R11 * V.he;
-                const float cfl = cost_at<TEX>(T, icx, fcx, icy, fcy, ofx + lx, ofy + ly, off);
-                const float cfr = cost_at<TEX>(T, icx, fcx, icy, fcy, ofx - lx, ofy - ly, off);
-                const float crl = cost_at<TEX>(T, icx, fcx, icy, fcy, orx + lx, ory + ly, off);
-                const float crr = cost_at<TEX>(T, icx, fcx, icy, fcy, orx - lx, ory - ly, off);
+                const float cfl = lookup<TEX>(T, cx, cy, base, ofx + lx, ofy + ly, off).w;
+                const float cfr = lookup<TEX>(T, cx, cy, base, ofx - lx, ofy - ly, off).w;
+                const float crl = lookup<TEX>(T, cx, cy, base, orx + lx, ory + ly, off).w;
+                const float crr = lookup<TEX>(T, cx, cy, base, orx - lx, ory - ly, off).w;
                 csum = (cfl + cfr) + (crl + crr);
             }
             const float soft = fmaxf(fmaf(-m, Cc.inv_eps, 1.f), 0.f);

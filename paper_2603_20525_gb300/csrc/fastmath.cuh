@@ -76,6 +76,30 @@ __device__ __forceinline__ void sincos_r(float x, float &s, float &c)
     c = (q == 0) ? cr : (q == 1) ? -sr : (q == 2) ? -cr : sr;
 }
 
+// sincos_r without the branch around the reduction: for |x| <= pi/4 the
+// quadrant is 0 and the reduction returns x itself, so the bits are
+// sincos_r's.  The quadrant comes from the low mantissa bits of a sum with
+// 1.5 x 2^23, not from a conversion.  SLOW = false leaves out CUDA's sincosf
+// for |x| >= kSincosMax: the caller tests for it and repeats with SLOW.
+constexpr float kSincosMax = 131072.f;
+template <bool SLOW>
+__device__ __forceinline__ void sincos_g(float x, float &s, float &c)
+{
+    const float t = __fadd_rn(x * 6.36619747e-01f, 12582912.f); // rint(x / (pi/2)) in the low bits
+    const float k = t - 12582912.f;
+    float r = fmaf(-k, 1.57079637e+00f, x);
+    r = fmaf(-k, -4.37113883e-08f, r);
+    r = fmaf(-k, -1.71512451e-15f, r);
+    float sr, cr;
+    sincos_q(r, sr, cr);
+    const unsigned q = __float_as_uint(t);
+    const bool odd = q & 1u;
+    s = __uint_as_float(__float_as_uint(odd ? cr : sr) ^ ((q & 2u) << 30));
+    c = __uint_as_float(__float_as_uint(odd ? sr : cr) ^ (((q + 1u) & 2u) << 30));
+    if (SLOW && fabsf(x) >= kSincosMax) sincosf(x, &s, &c);
+}
+__device__ __forceinline__ void sincos_b(float x, float &s, float &c) { sincos_g<true>(x, s, c); }
+
 // atan(r) for r in [0, 1] as r P(r^2), P of degree 8 fitted for minimum
 // maximum relative error (fit_atan.py): 1.1e-7 including FP32 evaluation.
 __device__ __forceinline__ float atan01(float r)

@@ -2,19 +2,16 @@
 // (arxiv 2603.20525, Sec. IV-A..IV-D) for sm_103a.
 //
 // Design
-//   * One, two or four threads per candidate (by batch size): a quad runs one
-//     wheel per lane and a pair one axle per lane, repeating the body
-//     arithmetic on every lane, so that small batches still give each SM
-//     sub-partition several warps.  The state stays in registers for the
-//     whole horizon; per Euler step the only memory traffic is 16 terrain
-//     texels (four bilinear lookups of one float4 per corner) through the
-//     read-only path, which the L1 and the 129 MB L2 serve for every terrain
-//     size used.
-//   * The arithmetic forms that measured faster in only some layouts are
-//     compile-time choices that give the same bits: the running cost's
-//     accumulator (FP32 or FP64), packed two-wide FP32 pairs and a goal
-//     test that discards the step rather than branching (two lanes), and
-//     loading each control one interval ahead (four lanes).
+//   * A full GPU runs one thread per candidate (rollout_one).  Below that the
+//     time is one candidate's chain of dependent instructions, and two warps
+//     share a group of candidates (the two-warp layouts below), with one, two
+//     or four lanes of each warp per candidate by batch size.  The state
+//     stays in registers for the whole horizon; per Euler step the only
+//     global memory traffic is 16 terrain texels (four bilinear lookups of
+//     one float4 per corner) through the read-only path, which the L1 and the
+//     129 MB L2 serve for every terrain size used.
+//   * Every layout forms every quantity by the same expressions in the same
+//     order, so all of them give the same bits.
 //   * Controls are time-major float2 [H][N]: a warp reads one coalesced 256 B
 //     line per control step.
 //   * The reduction is fused into the tail: a warp-shuffle min of a packed
@@ -31,43 +28,22 @@
 
 namespace atp {
 
-// Sum of v over the two lanes of a candidate's pair (a0 + a1 in both).
-__device__ __forceinline__ float pair_sum(float v, unsigned mask)
-{
-    return v + __shfl_xor_sync(mask, v, 1);
-}
-
-// One candidate per LANES consecutive threads.  LANES = 1: a thread runs all
-// four wheels.  LANES = 2: lane 0 runs the front axle's two wheels, lane 1
-// the rear's; each sums its axle, then one xor-shuffle per sum gives both
-// the same totals, in the same order as one lane computes them, so one and
-// two lanes give the same bits.  LANES = 4: lane q of the quad runs wheel q
-// (fl, fr, rl, rr) and forms the axle sums, then the totals, in that order
-// too, so all three layouts give the same bits.  The body-level arithmetic is repeated bit-identically on
-// every lane of a candidate, so lanes never exchange state, only the five
-// force/moment sums and the costmap sum, and the step's four sincos, which
-// the lanes split between them.  ACC selects the running cost's
-// accumulator: kAccF32, kAccF64, or kAccRuntime (p.acc64 decides; the batch
-// kernel, which would otherwise inline twice as many variants).  A
-// compile-time choice keeps the step loop free of the uniform branch.
+// ACC selects the running cost's accumulator: kAccF32, kAccF64, or
+// kAccRuntime (p.acc64 decides; the batch kernel, which would otherwise inline
+// twice as many variants).  A compile-time choice keeps the step loop free of
+// the uniform branch.
 constexpr int kAccF32 = 0, kAccF64 = 1, kAccRuntime = 2;
 
-
-template <int LANES, bool PER_X0, int TEX, int ACC>
-__device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, unsigned qmask,
-                                            float &J, float &margin, bool &feasible)
+// One thread per candidate.  The heading's sincos takes the reduction without
+// a branch (headings spread over the circle, so a warp ran both paths); roll,
+// pitch and steering stay mostly below pi/4 and keep it.
+template <bool PER_X0, int TEX, int ACC>
+__device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J, float &margin, bool &feasible)
 {
     const Veh &V = p.V;
     const Cost &Cc = p.C;
     const Terrain &T = p.T;
     {
-        // this lane's wheel (LANES = 4) or axle (LANES = 2)
-        const bool front = LANES == 2 ? q == 0 : q < 2;
-        const float wrx = front ? V.Lf : -V.Lr;
-        const float wry = (q & 1) ? -V.he : V.he;
-        const float wk = front ? V.kf : V.kr;
-        const float wb = front ? V.bf : V.br;
-        const float wFs = front ? V.Fsf : V.Fsr;
         // state; x, y relative to the terrain origin; *_l are the low parts of
         // the compensated components
         float x, xl, y, yl, z, zl, psi, psil, vx, vxl, vy, vyl, vz, vzl;
@@ -101,20 +77,12 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
         float msm = CUDART_INF_F, last_sm = CUDART_INF_F;
         int mstep = 0;
 
-        // four lanes load each interval's control one interval ahead, so the
-        // load's latency overlaps the Euler steps (measured faster there; one
-        // and two lanes run at the 128-register cap, where the two extra live
-        // registers cost more than the latency saved)
-        constexpr bool kPrefetch = LANES == 4;
-        float2 un = kPrefetch && p.H > 0 ? __ldg(p.ctrl + j) : make_float2(0.f, 0.f);
         for (int k = 0; k < p.H; ++k) {
             // zero-order hold; admissible steering rate |delta_dot| <= max
-            const float2 u = kPrefetch ? un : __ldg(p.ctrl + (size_t)k * p.N + j);
-            if (kPrefetch && k + 1 < p.H) un = __ldg(p.ctrl + (size_t)(k + 1) * p.N + j);
-            // one and two lanes ask L1 for the next interval's control instead,
-            // which costs no register (measured 3.6 % off the 16384-candidate
-            // plan, no change to a full-GPU plan)
-            if (!kPrefetch && k + 1 < p.H)
+            const float2 u = __ldg(p.ctrl + (size_t)k * p.N + j);
+            // ask L1 for the next interval's control, which costs no register
+            // (holding it in one costs more here than the latency saved)
+            if (k + 1 < p.H)
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(p.ctrl + (size_t)(k + 1) * p.N + j));
             const float dd = clamp_keep_nan(u.x, -V.ddmax, V.ddmax);
             const float ax = u.y;
@@ -124,175 +92,71 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
                     sm = fminf(sm, Ufrozen);
                     continue;
                 }
-                // four lanes split the step's four sincos (psi, theta, phi,
-                // delta; one each) and two lanes split them two and two,
-                // exchanging them by shuffle: the same bits as computing all
-                // four (measured 8 % off a 16384-candidate plan with four
-                // lanes, 2.4 % with two)
-                float sps, cps, sth, cth, sph, cph, cdl = 1.f;
-                if constexpr (LANES == 4) {
-                    float s1, c1;
-                    sincos_r(q == 0 ? psi : q == 1 ? th : q == 2 ? ph : d, s1, c1);
-                    sps = __shfl_sync(qmask, s1, 0, 4);
-                    cps = __shfl_sync(qmask, c1, 0, 4);
-                    sth = __shfl_sync(qmask, s1, 1, 4);
-                    cth = __shfl_sync(qmask, c1, 1, 4);
-                    sph = __shfl_sync(qmask, s1, 2, 4);
-                    cph = __shfl_sync(qmask, c1, 2, 4);
-                    cdl = __shfl_sync(qmask, c1, 3, 4);
-                } else if constexpr (LANES == 2) {
-                    // lane 0: psi and phi; lane 1: theta and delta
-                    float s1, c1, s2, c2;
-                    sincos_r(q == 0 ? psi : th, s1, c1);
-                    sincos_r(q == 0 ? ph : d, s2, c2);
-                    const float os1 = __shfl_xor_sync(qmask, s1, 1), oc1 = __shfl_xor_sync(qmask, c1, 1);
-                    const float os2 = __shfl_xor_sync(qmask, s2, 1), oc2 = __shfl_xor_sync(qmask, c2, 1);
-                    sps = q == 0 ? s1 : os1;
-                    cps = q == 0 ? c1 : oc1;
-                    sth = q == 0 ? os1 : s1;
-                    cth = q == 0 ? oc1 : c1;
-                    sph = q == 0 ? s2 : os2;
-                    cph = q == 0 ? c2 : oc2;
-                    cdl = q == 0 ? oc2 : c2;
-                } else {
-                    sincos_r(psi, sps, cps);
-                    sincos_r(th, sth, cth);
-                    sincos_r(ph, sph, cph);
-                }
+                float sps, cps, sth, cth, sph, cph;
+                sincos_b(psi, sps, cps);
+                sincos_r(th, sth, cth);
+                sincos_r(ph, sph, cph);
                 const float U = esm(V, ph, sph, cph, cth);
                 margin = fminf(margin, U);
                 sm = fminf(sm, U);
-                // goal test before the step (Sec. IV-C, reading Q4).  One and
-                // four lanes skip the step at the goal; two lanes compute it
-                // and discard it (`keep`), which keeps the loop body one basic
-                // block and measured faster there, slower with one or four
+                // goal test before the step (Sec. IV-C, reading Q4)
                 const float gdx = (x - Cc.gx_hi) + (xl - Cc.gx_lo);
                 const float gdy = (y - Cc.gy_hi) + (yl - Cc.gy_lo);
-                const bool reached = fmaf(gdx, gdx, gdy * gdy) <= Cc.goal_r2;
-                if (LANES != 2 && reached) {
+                if (fmaf(gdx, gdx, gdy * gdy) <= Cc.goal_r2) {
                     done = true;
                     Ufrozen = U;
                     continue;
                 }
-                const bool keep = LANES == 2 && reached;
-                bool offs = false;     // a wheel of this step off the map
                 // 3-2-1 rotation, body -> world (Sec. IV-A)
                 Body B;
                 float *R = B.R;
                 R[0] = cps * cth;
-                if constexpr (LANES == 2) {
-                    // packed pairs, the same bits (see wheel's PAIRED)
-                    const float2 r12 = fma2(make_float2(cps * sph, cph * cps), splat2(sth),
-                                            make_float2(-cph * sps, sph * sps));
-                    const float2 r45 = fma2(make_float2(sph * sps, cph * sps), splat2(sth),
-                                            make_float2(cph * cps, -cps * sph));
-                    R[1] = r12.x; R[2] = r12.y; R[4] = r45.x; R[5] = r45.y;
-                } else {
-                    R[1] = fmaf(cps * sph, sth, -cph * sps);
-                    R[2] = fmaf(cph * cps, sth, sph * sps);
-                    R[4] = fmaf(sph * sps, sth, cph * cps);
-                    R[5] = fmaf(cph * sps, sth, -cps * sph);
-                }
+                R[1] = fmaf(cps * sph, sth, -cph * sps);
+                R[2] = fmaf(cph * cps, sth, sph * sps);
+                R[4] = fmaf(sph * sps, sth, cph * cps);
+                R[5] = fmaf(cph * sps, sth, -cps * sph);
                 R[3] = cth * sps;
                 R[6] = -sth;
                 R[7] = cth * sph;
                 R[8] = cph * cth;
-                cell_split(x, xl, T.inv_cell, B.icx, B.fcx);
-                cell_split(y, yl, T.inv_cell, B.icy, B.fcy);
+                B.cx = cell_of(x, xl, T.inv_cell, T.nx);
+                B.cy = cell_of(y, yl, T.inv_cell, T.ny);
+                B.base = texel_base(B.cx, B.cy, T.nx);
+                off = off || off_com(B.cx, B.cy);
                 B.z_hi = z;
                 B.z_lo = zl;
                 B.vx = vx; B.vy = vy; B.vz = vz;
                 B.wx = wx; B.wy = wy; B.wz = wz;
                 // gravity in B: R^T (0, 0, -g)
                 const float gBx = -V.g * R[6], gBy = -V.g * R[7], gBz = -V.g * R[8];
-                float cd;
-                if constexpr (LANES > 1) {
-                    cd = cdl;
-                } else {
-                    float sd;
-                    sincos_r(d, sd, cd);
-                }
+                float sd, cd;
+                sincos_r(d, sd, cd);
                 // summed forces and moments (Sec. IV-A); the rear
                 // longitudinal constraint force enters My only
-                float FyB, FzB, Mx, My, Mz, csum;
-                if (LANES == 1) {
-                    const WheelOut fl = wheel<TEX>(V, T, B, V.Lf, V.he, V.kf, V.bf, V.Fsf, d, offs);
-                    const WheelOut fr = wheel<TEX>(V, T, B, V.Lf, -V.he, V.kf, V.bf, V.Fsf, d, offs);
-                    const WheelOut rl = wheel<TEX>(V, T, B, -V.Lr, V.he, V.kr, V.br, V.Fsr, 0.f, offs);
-                    const WheelOut rr = wheel<TEX>(V, T, B, -V.Lr, -V.he, V.kr, V.br, V.Fsr, 0.f, offs);
-                    const float Fyf = (fl.Fy + fr.Fy) * cd;
-                    const float Fyr = rl.Fy + rr.Fy;
-                    FyB = Fyf + Fyr;
-                    FzB = (fl.Fz + fr.Fz) + (rl.Fz + rr.Fz);
-                    Mx = fmaf(V.hR, FyB, V.he * ((fl.Fz - fr.Fz) + (rl.Fz - rr.Fz)));
-                    My = -V.Lf * (fl.Fz + fr.Fz) + V.Lr * (rl.Fz + rr.Fz);
-                    Mz = V.Lf * Fyf + -V.Lr * Fyr;
-                    csum = (fl.cost + fr.cost) + (rl.cost + rr.cost);
-                } else if (LANES == 2) {
-                    // this lane's axle: left and right wheel
-                    const float di = front ? d : 0.f;
-                    const WheelOut l = wheel<TEX, true>(V, T, B, wrx, V.he, wk, wb, wFs, di, offs);
-                    const WheelOut r = wheel<TEX, true>(V, T, B, wrx, -V.he, wk, wb, wFs, di, offs);
-                    const float fy = front ? (l.Fy + r.Fy) * cd : l.Fy + r.Fy;
-                    const float fz = l.Fz + r.Fz;
-                    FyB = pair_sum(fy, qmask);
-                    FzB = pair_sum(fz, qmask);
-                    Mx = fmaf(V.hR, FyB, V.he * pair_sum(l.Fz - r.Fz, qmask));
-                    My = pair_sum(-wrx * fz, qmask);
-                    Mz = pair_sum(wrx * fy, qmask);
-                    csum = T.has_cm ? pair_sum(l.cost + r.cost, qmask) : 0.f;
-                } else {
-                    // this lane's wheel; its axle's sums by one xor-shuffle,
-                    // the other axle's by a second, each formed in the order
-                    // one lane forms it (a + b is b + a; the differences and
-                    // the moments pick their operands by lane), so four lanes
-                    // give the bits of one and two
-                    const WheelOut w = wheel<TEX>(V, T, B, wrx, wry, wk, wb, wFs, front ? d : 0.f, offs);
-                    const bool left = (q & 1) == 0;
-                    const float oFy = __shfl_xor_sync(qmask, w.Fy, 1);
-                    const float oFz = __shfl_xor_sync(qmask, w.Fz, 1);
-                    const float aFy = w.Fy + oFy;
-                    const float afy = front ? aFy * cd : aFy;                  // Fyf or Fyr
-                    const float aFz = w.Fz + oFz;
-                    const float aDz = left ? w.Fz - oFz : oFz - w.Fz;           // left - right
-                    const float bfy = __shfl_xor_sync(qmask, afy, 2);
-                    const float bFz = __shfl_xor_sync(qmask, aFz, 2);
-                    const float bDz = __shfl_xor_sync(qmask, aDz, 2);
-                    const float Fyf = front ? afy : bfy, Fyr = front ? bfy : afy;
-                    const float Fzf = front ? aFz : bFz, Fzr = front ? bFz : aFz;
-                    FyB = Fyf + Fyr;
-                    FzB = Fzf + Fzr;
-                    Mx = fmaf(V.hR, FyB, V.he * (aDz + bDz));
-                    My = -V.Lf * Fzf + V.Lr * Fzr;
-                    Mz = V.Lf * Fyf + -V.Lr * Fyr;
-                    if (T.has_cm) {
-                        const float ac = w.cost + __shfl_xor_sync(qmask, w.cost, 1);
-                        csum = ac + __shfl_xor_sync(qmask, ac, 2);
-                    } else {
-                        csum = 0.f;
-                    }
-                }
+                const WheelOut fl = wheel<TEX>(V, T, B, V.Lf, V.he, V.kf, V.bf, V.Fsf, d, off);
+                const WheelOut fr = wheel<TEX>(V, T, B, V.Lf, -V.he, V.kf, V.bf, V.Fsf, d, off);
+                const WheelOut rl = wheel<TEX>(V, T, B, -V.Lr, V.he, V.kr, V.br, V.Fsr, 0.f, off);
+                const WheelOut rr = wheel<TEX>(V, T, B, -V.Lr, -V.he, V.kr, V.br, V.Fsr, 0.f, off);
+                const float Fyf = (fl.Fy + fr.Fy) * cd;
+                const float Fyr = rl.Fy + rr.Fy;
+                const float FyB = Fyf + Fyr;
+                const float FzB = (fl.Fz + fr.Fz) + (rl.Fz + rr.Fz);
+                const float Mx = fmaf(V.hR, FyB, V.he * ((fl.Fz - fr.Fz) + (rl.Fz - rr.Fz)));
+                float My = -V.Lf * (fl.Fz + fr.Fz) + V.Lr * (rl.Fz + rr.Fz);
+                const float Mz = V.Lf * Fyf + -V.Lr * Fyr;
+                const float csum = (fl.cost + fr.cost) + (rl.cost + rr.cost);
                 const float Fx = V.halfM * fmaf(-wz, vy, fmaf(wy, vz, ax - gBx));
                 My = fmaf(-V.hR, 2.f * Fx, My);
                 // running cost L = L_0 + L_soft (Sec. IV-C), left Riemann sum
                 const float soft = fmaxf(fmaf(-U, Cc.inv_eps, 1.f), 0.f);
                 const float L = fmaf(Cc.sigma * soft, soft, fmaf(Cc.wc * dd, dd, Cc.wt)) + csum;
-                if (acc64) J64 += keep ? 0.0 : (double)(h * L);
-                else J = keep ? J : fmaf(h, L, J);
+                if (acc64) J64 += (double)(h * L);
+                else J = fmaf(h, L, J);
                 // state derivative A(xi) + B zeta (Sec. IV-A)
                 const float ic = rcp(cth);
                 const float wsc = fmaf(sph, wy, cph * wz);
-                float dx, dy;
-                if constexpr (LANES == 2) {
-                    const float2 dxy = fma2(make_float2(R[2], R[5]), splat2(vz),
-                                            fma2(make_float2(R[1], R[4]), splat2(vy),
-                                                 make_float2(R[0] * vx, R[3] * vx)));
-                    dx = dxy.x;
-                    dy = dxy.y;
-                } else {
-                    dx = fmaf(R[2], vz, fmaf(R[1], vy, R[0] * vx));
-                    dy = fmaf(R[5], vz, fmaf(R[4], vy, R[3] * vx));
-                }
+                const float dx = fmaf(R[2], vz, fmaf(R[1], vy, R[0] * vx));
+                const float dy = fmaf(R[5], vz, fmaf(R[4], vy, R[3] * vx));
                 const float dz = fmaf(R[8], vz, fmaf(R[7], vy, R[6] * vx));
                 const float dpsi = wsc * ic;
                 const float dth = fmaf(cph, wy, -sph * wz);
@@ -302,31 +166,22 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
                 const float dwx = fmaf(V.dJyz * wy, wz, Mx) * V.invJxx;
                 const float dwy = fmaf(-V.dJxz * wx, wz, My) * V.invJyy;
                 const float dwz = fmaf(V.dJxy * wx, wy, Mz) * V.invJzz;
-                // forward Euler (Sec. IV-D), steering angle clamped (reading Q5),
-                // committed unless the step is discarded at the goal
-                float nx = x, nxl = xl, ny = y, nyl = yl, nz = z, nzl = zl, np_ = psi, npl = psil;
-                float nvx = vx, nvxl = vxl, nvy = vy, nvyl = vyl, nvz = vz, nvzl = vzl;
-                acc2(nx, nxl, h * dx);
-                acc2(ny, nyl, h * dy);
-                acc2(nz, nzl, h * dz);
-                acc2(np_, npl, h * dpsi);
-                acc2(nvx, nvxl, h * ax);
-                acc2(nvy, nvyl, h * dvy);
-                acc2(nvz, nvzl, h * dvz);
-                const float nth = fmaf(h, dth, th), nph = fmaf(h, dph, ph);
-                const float nwx = fmaf(h, dwx, wx), nwy = fmaf(h, dwy, wy), nwz = fmaf(h, dwz, wz);
-                const float nd = clamp_keep_nan(fmaf(h, dd, d), -V.dmax, V.dmax);
-                if (!keep) {
-                    x = nx; xl = nxl; y = ny; yl = nyl; z = nz; zl = nzl; psi = np_; psil = npl;
-                    vx = nvx; vxl = nvxl; vy = nvy; vyl = nvyl; vz = nvz; vzl = nvzl;
-                    th = nth; ph = nph; wx = nwx; wy = nwy; wz = nwz; d = nd;
-                    off = off || offs;
-                } else {
-                    done = true;
-                    Ufrozen = U;
-                }
+                // forward Euler (Sec. IV-D), steering angle clamped (reading Q5)
+                acc2(x, xl, h * dx);
+                acc2(y, yl, h * dy);
+                acc2(z, zl, h * dz);
+                acc2(psi, psil, h * dpsi);
+                acc2(vx, vxl, h * ax);
+                acc2(vy, vyl, h * dvy);
+                acc2(vz, vzl, h * dvz);
+                th = fmaf(h, dth, th);
+                ph = fmaf(h, dph, ph);
+                wx = fmaf(h, dwx, wx);
+                wy = fmaf(h, dwy, wy);
+                wz = fmaf(h, dwz, wz);
+                d = clamp_keep_nan(fmaf(h, dd, d), -V.dmax, V.dmax);
             }
-            if (p.step_margin && q == 0 && k + 1 < p.H) p.step_margin[(size_t)k * p.N + j] = sm;
+            if (p.step_margin && k + 1 < p.H) p.step_margin[(size_t)k * p.N + j] = sm;
             if (k + 1 < p.H) {
                 if (sm < msm) {
                     msm = sm;
@@ -335,10 +190,6 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
             } else {
                 last_sm = sm;
             }
-        }
-        if (LANES > 1) {
-            // the off-map flag is per wheel: OR it over the candidate's lanes
-            off = __any_sync(qmask, off);
         }
         // final state: margin, goal test, terminal cost Phi (Sec. IV-C)
         {
@@ -349,7 +200,7 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
             margin = fminf(margin, U);
             last_sm = fminf(last_sm, U);
             if (last_sm < msm) mstep = p.H - 1;
-            if (p.step_margin && q == 0) p.step_margin[(size_t)(p.H - 1) * p.N + j] = last_sm;
+            if (p.step_margin) p.step_margin[(size_t)(p.H - 1) * p.N + j] = last_sm;
             const float gdx = (x - Cc.gx_hi) + (xl - Cc.gx_lo);
             const float gdy = (y - Cc.gy_hi) + (yl - Cc.gy_lo);
             const float d2 = fmaf(gdx, gdx, gdy * gdy);
@@ -366,42 +217,502 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, int q, u
         for (int c = 0; c < 13; ++c) finite = finite && isfinite(xs[c]);
         if (!finite) J = CUDART_INF_F;
         feasible = finite && margin > 0.f;
-        if (q == 0) {
-            const uint8_t fl = (feasible ? ATP_FLAG_FEASIBLE : 0) | (done ? ATP_FLAG_DONE : 0) |
-                               (off ? ATP_FLAG_OFFMAP : 0) | (finite ? 0 : ATP_FLAG_NONFINITE);
-            if (p.cost) p.cost[j] = J;
-            if (p.margin) p.margin[j] = margin;
-            if (p.flags) p.flags[j] = fl;
-            if (p.min_step) p.min_step[j] = mstep;
-            if (p.xf) {
-                const size_t N = (size_t)p.N;
+        const uint8_t fl = (feasible ? ATP_FLAG_FEASIBLE : 0) | (done ? ATP_FLAG_DONE : 0) |
+                           (off ? ATP_FLAG_OFFMAP : 0) | (finite ? 0 : ATP_FLAG_NONFINITE);
+        if (p.cost) p.cost[j] = J;
+        if (p.margin) p.margin[j] = margin;
+        if (p.flags) p.flags[j] = fl;
+        if (p.min_step) p.min_step[j] = mstep;
+        if (p.xf) {
+            const size_t N = (size_t)p.N;
 #pragma unroll
-                for (int c = 0; c < 13; ++c) p.xf[c * N + j] = xs[c];
-            }
+            for (int c = 0; c < 13; ++c) p.xf[c * N + j] = xs[c];
         }
     }
 
 }
 
-// Register budgets, from A/B runs on the GB300: four lanes run best with
-// ptxas free to use about 104 registers (minimum 1 CTA per SM), one and two
-// lanes with the 128-register cap of 8 resident 64-thread CTAs per SM.
-template <int LANES, bool PER_X0, bool REDUCE, int TEX, int ACC>
-__global__ void __launch_bounds__(kPlanBlock, LANES == 4 ? 1 : 8)
+// Five CTAs per SM leave ptxas 168 registers and no spills: 4.75 ms on the
+// paper configuration against 4.84 ms at six and 4.87 ms at seven (128
+// registers, 32 B of spills; the lookups' map edges keep more values live
+// than the integer clamps they replaced).
+template <bool PER_X0, bool REDUCE, int TEX, int ACC>
+__global__ void __launch_bounds__(kPlanBlock, 5)
 plan_kernel(const __grid_constant__ PlanParams p)
 {
-    // 64-bit: N x LANES threads may exceed 2^31 when the lanes are forced
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = (int)(tid / LANES);
-    const int q = LANES == 1 ? 0 : (int)(tid & (LANES - 1));
+    const int j = blockIdx.x * kPlanBlock + threadIdx.x;     // N <= 2^31 - 1025
     const bool live = j < p.N;
-    const unsigned qmask = LANES == 1 ? 0u : LANES == 2 ? (0x3u << (threadIdx.x & 30))
-                                                        : (0xfu << (threadIdx.x & 28));
     float J = 0.f, margin = CUDART_INF_F;
     bool feasible = false;
-    if (live) rollout_one<LANES, PER_X0, TEX, ACC>(p, j, q, qmask, J, margin, feasible);
+    if (live) rollout_one<PER_X0, TEX, ACC>(p, j, J, margin, feasible);
     if (!REDUCE) return;
-    plan_tail(p, j, live && q == 0, J, feasible, gridDim.x);
+    plan_tail(p, j, live, J, feasible, gridDim.x);
+}
+
+// ---- two warps per group of candidates ------------------------------------
+//
+// Forward Euler moves position and attitude with the velocities of the step's
+// start, so the lookups of step t + 1 do not wait for the forces of step t.
+// In each pair of warps one ("geometry") advances position, attitude and
+// steering and looks the terrain up, and the other ("forces") turns the
+// geometry of step t into the velocities of step t + 1, and accumulates the
+// cost and the margins, while the first is at the geometry of step t + 1.
+// They swap through shared memory (two buffers) with one CTA barrier per Euler
+// step:
+//
+//   slot t    geometry warp: v(t) -> state(t+1) -> geometry(t+1)
+//             forces warp:   geometry(t), v(t) -> v(t+1)
+//
+// Every quantity is formed by the same expressions as in one thread, so the
+// bits are the same.
+template <int LANES>
+struct Duo {
+    static constexpr int kW = 4 / LANES;            // wheels per lane
+    static constexpr int kC = 32 / LANES;           // candidates per pair of warps
+    float4 tau[2][kW][32];                          // tx, ty, tz, 1 / tz per wheel
+    float2 chi[2][kW][32];                          // extension, costmap
+    float4 att[2][kC];                              // sin and cos of theta, then of phi
+    float4 body[2][kC];                             // delta, cos(delta), phi; done (0 or 1)
+    float4 va[2][kC];                               // vx, vy, vz, wx
+    float2 vb[2][kC];                               // wy, wz
+    float d2[kC];                                   // final squared distance to the goal
+    int flags[kC];                                  // done, off the map, final state not finite
+    int flip;                                       // which warp takes which role
+};
+
+constexpr unsigned kFull = 0xffffffffu;
+
+// c ? a : b as a select: the compiler turns chains of conditionals on the
+// lane into divergent branches, which cost far more than the selects
+__device__ __forceinline__ float sel(bool c, float a, float b)
+{
+    float r;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %3, 0;\n\tselp.f32 %0, %1, %2, p;\n\t}" : "=f"(r) : "f"(a), "f"(b), "r"((int)c));
+    return r;
+}
+__device__ __forceinline__ void pair_barrier() { asm volatile("bar.sync 0;" ::: "memory"); }
+
+// this lane's first wheel or axle
+struct LaneWheel {
+    bool front;
+    float rx, ry, k, b, Fs;
+};
+template <int LANES>
+__device__ __forceinline__ LaneWheel lane_wheel(const Veh &V, int q)
+{
+    LaneWheel w;
+    w.front = LANES == 1 || (LANES == 2 ? q == 0 : q < 2);
+    w.rx = w.front ? V.Lf : -V.Lr;
+    w.ry = LANES < 4 ? V.he : (q & 1) ? -V.he : V.he;
+    w.k = w.front ? V.kf : V.kr;
+    w.b = w.front ? V.bf : V.br;
+    w.Fs = w.front ? V.Fsf : V.Fsr;
+    return w;
+}
+
+// Sum of v over the two lanes of a candidate's pair (a0 + a1 in both).
+__device__ __forceinline__ float pair_sum(float v) { return v + __shfl_xor_sync(kFull, v, 1); }
+
+struct Fast { static constexpr bool value = false; };
+struct Slow { static constexpr bool value = true; };
+
+template <int LANES, bool PER_X0, int TEX>
+__device__ __forceinline__ void duo_geometry(const PlanParams &p, Duo<LANES> &sh, int j, int q, int c, bool live)
+{
+    const Veh &V = p.V;
+    const Cost &Cc = p.C;
+    const Terrain &T = p.T;
+    const int lane = threadIdx.x & 31;
+    const LaneWheel lw = lane_wheel<LANES>(V, q);
+    float x = 0.f, xl = 0.f, y = 0.f, yl = 0.f, z = 0.f, zl = 0.f, psi = 0.f, psil = 0.f, th = 0.f, ph = 0.f, d = 0.f;
+    if (live) {
+        const size_t N = (size_t)p.N;
+        const auto x0 = [&](int r) { return PER_X0 ? __ldg(p.x0_soa + r * N + j) : p.x0[r]; };
+        two_sum(x0(0), -T.x0_hi, x, xl);
+        xl -= T.x0_lo;
+        two_sum(x0(1), -T.y0_hi, y, yl);
+        yl -= T.y0_lo;
+        z = x0(2); psi = x0(3); th = x0(4); ph = x0(5); d = x0(12);
+    }
+    bool done = !live, off = false, offs = false;
+    const float h = p.h;
+    float R[9], sth = 0.f, cth = 1.f, sph = 0.f, cph = 1.f;
+    const bool q1 = (q & 1) != 0, q2 = (q & 2) != 0;
+    bool huge = false;               // an angle beyond the fast reduction
+
+    // the goal test and the wheels' geometry of the current state, into
+    // buffer `par`
+    const auto geometry = [&](int par, auto form) {
+        float sps, cps, cdl;
+        if constexpr (LANES == 4) {
+            float s1, c1;
+            const float an = sel(q2, sel(q1, d, ph), sel(q1, th, psi));
+            sincos_g<decltype(form)::value>(an, s1, c1);
+            huge = fabsf(an) >= kSincosMax;
+            sps = __shfl_sync(kFull, s1, 0, 4);
+            cps = __shfl_sync(kFull, c1, 0, 4);
+            sth = __shfl_sync(kFull, s1, 1, 4);
+            cth = __shfl_sync(kFull, c1, 1, 4);
+            sph = __shfl_sync(kFull, s1, 2, 4);
+            cph = __shfl_sync(kFull, c1, 2, 4);
+            cdl = __shfl_sync(kFull, c1, 3, 4);
+        } else if constexpr (LANES == 1) {
+            float sdl;
+            sincos_g<decltype(form)::value>(psi, sps, cps);
+            sincos_g<decltype(form)::value>(th, sth, cth);
+            sincos_g<decltype(form)::value>(ph, sph, cph);
+            sincos_g<decltype(form)::value>(d, sdl, cdl);
+            huge = fmaxf(fmaxf(fabsf(psi), fabsf(th)), fmaxf(fabsf(ph), fabsf(d))) >= kSincosMax;
+        } else {
+            // lane 0: psi and phi; lane 1: theta and delta
+            float s1, c1, s2, c2;
+            const float a1 = sel(q1, th, psi), a2 = sel(q1, d, ph);
+            sincos_g<decltype(form)::value>(a1, s1, c1);
+            sincos_g<decltype(form)::value>(a2, s2, c2);
+            huge = fmaxf(fabsf(a1), fabsf(a2)) >= kSincosMax;
+            const float os1 = __shfl_xor_sync(kFull, s1, 1), oc1 = __shfl_xor_sync(kFull, c1, 1);
+            const float os2 = __shfl_xor_sync(kFull, s2, 1), oc2 = __shfl_xor_sync(kFull, c2, 1);
+            sps = sel(q1, os1, s1);
+            cps = sel(q1, oc1, c1);
+            sth = sel(q1, s1, os1);
+            cth = sel(q1, c1, oc1);
+            sph = sel(q1, os2, s2);
+            cph = sel(q1, oc2, c2);
+            cdl = sel(q1, c2, oc2);
+        }
+        // 3-2-1 rotation, body -> world (Sec. IV-A)
+        R[0] = cps * cth;
+        R[1] = fmaf(cps * sph, sth, -cph * sps);
+        R[2] = fmaf(cph * cps, sth, sph * sps);
+        R[3] = cth * sps;
+        R[4] = fmaf(sph * sps, sth, cph * cps);
+        R[5] = fmaf(cph * sps, sth, -cps * sph);
+        R[6] = -sth;
+        R[7] = cth * sph;
+        R[8] = cph * cth;
+        // goal test before the step (Sec. IV-C, reading Q4)
+        const float gdx = (x - Cc.gx_hi) + (xl - Cc.gx_lo);
+        const float gdy = (y - Cc.gy_hi) + (yl - Cc.gy_lo);
+        done = done || fmaf(gdx, gdx, gdy * gdy) <= Cc.goal_r2;
+        if (q == 0) {
+            sh.att[par][c] = make_float4(sth, cth, sph, cph);
+            sh.body[par][c] = make_float4(d, cdl, ph, done ? 1.f : 0.f);
+        }
+        const Cell cx = cell_of(x, xl, T.inv_cell, T.nx), cy = cell_of(y, yl, T.inv_cell, T.ny);
+        const unsigned base = texel_base(cx, cy, T.nx);
+        offs = off_com(cx, cy);
+    #pragma unroll
+        for (int w = 0; w < Duo<LANES>::kW; ++w) {
+            const WheelGeo g = wheel_geo<TEX>(V, T, R, cx, cy, base, z, zl, w < 2 ? lw.rx : -V.Lr,
+                                              LANES == 4 ? lw.ry : (w & 1) ? -V.he : V.he, offs);
+            sh.tau[par][w][lane] = make_float4(g.tx, g.ty, g.tz, g.itz);
+            sh.chi[par][w][lane] = make_float2(g.chi, g.cost);
+        }
+    };
+
+    geometry(0, Fast{});
+    if (__any_sync(kFull, huge)) geometry(0, Slow{});
+    pair_barrier();
+    int par = 0;
+    float un = live ? __ldg(&p.ctrl[j].x) : 0.f;
+    for (int k = 0; k < p.H; ++k) {
+        // zero-order hold; admissible steering rate |delta_dot| <= max
+        const float dd = clamp_keep_nan(un, -V.ddmax, V.ddmax);
+        if (live && k + 1 < p.H) un = __ldg(&p.ctrl[(size_t)(k + 1) * p.N + j].x);
+        const bool idle = __all_sync(kFull, done);     // every candidate frozen at the goal
+        for (int sub = 0; sub < p.n_sub; ++sub) {
+            if (!idle) {
+                const float4 va = sh.va[par][c];
+                const float2 vb = sh.vb[par][c];
+                const float vx = va.x, vy = va.y, vz = va.z, wx = va.w, wy = vb.x, wz = vb.y;
+                const bool go = !done;
+                off = off || (go && offs);
+                // position, attitude and steering of A(xi) + B zeta (Sec. IV-A), forward Euler
+                const float ic = rcp(cth);
+                const float wsc = fmaf(sph, wy, cph * wz);
+                const float dx = fmaf(R[2], vz, fmaf(R[1], vy, R[0] * vx));
+                const float dy = fmaf(R[5], vz, fmaf(R[4], vy, R[3] * vx));
+                const float dz = fmaf(R[8], vz, fmaf(R[7], vy, R[6] * vx));
+                const float dpsi = wsc * ic;
+                const float dth = fmaf(cph, wy, -sph * wz);
+                const float dph = fmaf(wsc, sth * ic, wx);
+                float nx = x, nxl = xl, ny = y, nyl = yl, nz = z, nzl = zl, np_ = psi, npl = psil;
+                acc2(nx, nxl, h * dx);
+                acc2(ny, nyl, h * dy);
+                acc2(nz, nzl, h * dz);
+                acc2(np_, npl, h * dpsi);
+                const float nth = fmaf(h, dth, th), nph = fmaf(h, dph, ph);
+                const float nd = clamp_keep_nan(fmaf(h, dd, d), -V.dmax, V.dmax);
+                // frozen at the goal: the step is computed and discarded, which
+                // keeps the warp converged for the shuffles
+                x = sel(go, nx, x); xl = sel(go, nxl, xl); y = sel(go, ny, y); yl = sel(go, nyl, yl);
+                z = sel(go, nz, z); zl = sel(go, nzl, zl); psi = sel(go, np_, psi); psil = sel(go, npl, psil);
+                th = sel(go, nth, th); ph = sel(go, nph, ph); d = sel(go, nd, d);
+                geometry(par ^ 1, Fast{});
+                if (__any_sync(kFull, huge)) geometry(par ^ 1, Slow{});
+            }
+            pair_barrier();
+            par ^= 1;
+        }
+    }
+    // the off-map flag is per wheel: OR it over the candidate's lanes
+    const unsigned offm = __ballot_sync(kFull, off) >> (lane & ~(LANES - 1));
+    off = (offm & ((1u << LANES) - 1u)) != 0u;
+    // fold the low parts back and leave the terrain frame
+    const float xs[7] = {(x + T.x0_hi) + (xl + T.x0_lo), (y + T.y0_hi) + (yl + T.y0_lo), z + zl, psi + psil, th, ph,
+                         d};
+    if (q == 0) {
+        const float gdx = (x - Cc.gx_hi) + (xl - Cc.gx_lo);
+        const float gdy = (y - Cc.gy_hi) + (yl - Cc.gy_lo);
+        bool finite = true;
+#pragma unroll
+        for (int r = 0; r < 7; ++r) finite = finite && isfinite(xs[r]);
+        sh.d2[c] = fmaf(gdx, gdx, gdy * gdy);
+        sh.flags[c] = (done ? ATP_FLAG_DONE : 0) | (off ? ATP_FLAG_OFFMAP : 0) | (finite ? 0 : ATP_FLAG_NONFINITE);
+        if (live && p.xf) {
+            const size_t N = (size_t)p.N;
+#pragma unroll
+            for (int r = 0; r < 6; ++r) p.xf[r * N + j] = xs[r];
+            p.xf[12 * N + j] = xs[6];
+        }
+    }
+    pair_barrier();
+}
+
+template <int LANES, bool PER_X0, int ACC>
+__device__ __forceinline__ void duo_forces(const PlanParams &p, Duo<LANES> &sh, int j, int q, int c, bool live,
+                                           float &J, float &margin, bool &feasible)
+{
+    const Veh &V = p.V;
+    const Cost &Cc = p.C;
+    const int lane = threadIdx.x & 31;
+    const LaneWheel lw = lane_wheel<LANES>(V, q);
+    const bool front = lw.front, left = (q & 1) == 0;
+    float vx = 0.f, vxl = 0.f, vy = 0.f, vyl = 0.f, vz = 0.f, vzl = 0.f, wx = 0.f, wy = 0.f, wz = 0.f;
+    if (live) {
+        const size_t N = (size_t)p.N;
+        const auto x0 = [&](int r) { return PER_X0 ? __ldg(p.x0_soa + r * N + j) : p.x0[r]; };
+        vx = x0(6); vy = x0(7); vz = x0(8); wx = x0(9); wy = x0(10); wz = x0(11);
+    }
+    const float h = p.h;
+    const bool acc64 = ACC == kAccRuntime ? p.acc64 != 0 : ACC == kAccF64;
+    const bool cm = p.T.has_cm != 0;
+    double J64 = 0.0;
+    float U = 0.f, msm = CUDART_INF_F, last_sm = CUDART_INF_F;
+    int mstep = 0;
+    if (q == 0) {
+        sh.va[0][c] = make_float4(vx, vy, vz, wx);
+        sh.vb[0][c] = make_float2(wy, wz);
+    }
+    pair_barrier();
+    int par = 0;
+    bool idle = false;
+    float2 un = live ? __ldg(p.ctrl + j) : make_float2(0.f, 0.f);
+    for (int k = 0; k < p.H; ++k) {
+        const float dd = clamp_keep_nan(un.x, -V.ddmax, V.ddmax), ax = un.y;
+        if (live && k + 1 < p.H) un = __ldg(p.ctrl + (size_t)(k + 1) * p.N + j);
+        if (!idle) {
+            // for good: the geometry warp leaves the buffers as they are
+            const float4 att = sh.att[par][c], body = sh.body[par][c];
+            U = esm(V, body.z, att.z, att.w, att.y);
+            idle = __all_sync(kFull, body.w != 0.f);
+        }
+        float sm = CUDART_INF_F;
+        for (int sub = 0; sub < p.n_sub; ++sub) {
+            if (!idle) {
+                const float4 att = sh.att[par][c], body = sh.body[par][c];
+                const float sth = att.x, cth = att.y, sph = att.z, cph = att.w, cd = body.y;
+                const float di = front ? body.x : 0.f;
+                const bool go = body.w == 0.f;
+                // gravity in B: R^T (0, 0, -g)
+                const float gBx = -V.g * -sth, gBy = -V.g * (cth * sph), gBz = -V.g * (cph * cth);
+                // summed forces and moments (Sec. IV-A); the rear
+                // longitudinal constraint force enters My only
+                float FyB, FzB, Mx, My, Mz, csum = 0.f;
+                const float4 t0 = sh.tau[par][0][lane];
+                const float2 x0 = sh.chi[par][0][lane];
+                const WheelGeo g0 = {t0.x, t0.y, t0.z, t0.w, x0.x, x0.y};
+                if constexpr (LANES == 1) {
+                    const auto wh = [&](int i, float rx, float ry, float k, float b, float Fs, float dw) {
+                        const float4 t = sh.tau[par][i][lane];
+                        const float2 x = sh.chi[par][i][lane];
+                        const WheelGeo g = {t.x, t.y, t.z, t.w, x.x, x.y};
+                        return wheel_dyn(V, g, vx, vy, vz, wx, wy, wz, rx, ry, k, b, Fs, dw);
+                    };
+                    const WheelOut fl = wh(0, V.Lf, V.he, V.kf, V.bf, V.Fsf, di), fr = wh(1, V.Lf, -V.he, V.kf, V.bf, V.Fsf, di);
+                    const WheelOut rl = wh(2, -V.Lr, V.he, V.kr, V.br, V.Fsr, 0.f), rr = wh(3, -V.Lr, -V.he, V.kr, V.br, V.Fsr, 0.f);
+                    const float Fyf = (fl.Fy + fr.Fy) * cd;
+                    const float Fyr = rl.Fy + rr.Fy;
+                    FyB = Fyf + Fyr;
+                    FzB = (fl.Fz + fr.Fz) + (rl.Fz + rr.Fz);
+                    Mx = fmaf(V.hR, FyB, V.he * ((fl.Fz - fr.Fz) + (rl.Fz - rr.Fz)));
+                    My = -V.Lf * (fl.Fz + fr.Fz) + V.Lr * (rl.Fz + rr.Fz);
+                    Mz = V.Lf * Fyf + -V.Lr * Fyr;
+                    csum = (fl.cost + fr.cost) + (rl.cost + rr.cost);
+                } else if constexpr (LANES == 2) {
+                    const float4 t1 = sh.tau[par][1][lane];
+                    const float2 x1 = sh.chi[par][1][lane];
+                    const WheelGeo g1 = {t1.x, t1.y, t1.z, t1.w, x1.x, x1.y};
+                    const WheelOut l = wheel_dyn<true>(V, g0, vx, vy, vz, wx, wy, wz, lw.rx, V.he, lw.k, lw.b, lw.Fs, di);
+                    const WheelOut r = wheel_dyn<true>(V, g1, vx, vy, vz, wx, wy, wz, lw.rx, -V.he, lw.k, lw.b, lw.Fs, di);
+                    const float fy = sel(front, (l.Fy + r.Fy) * cd, l.Fy + r.Fy);
+                    const float fz = l.Fz + r.Fz;
+                    FyB = pair_sum(fy);
+                    FzB = pair_sum(fz);
+                    Mx = fmaf(V.hR, FyB, V.he * pair_sum(l.Fz - r.Fz));
+                    My = pair_sum(-lw.rx * fz);
+                    Mz = pair_sum(lw.rx * fy);
+                    if (cm) csum = pair_sum(l.cost + r.cost);
+                } else {
+                    // the axle's sums by one xor-shuffle, the other axle's by a
+                    // second, each formed in the order one lane forms it
+                    const WheelOut w = wheel_dyn(V, g0, vx, vy, vz, wx, wy, wz, lw.rx, lw.ry, lw.k, lw.b, lw.Fs, di);
+                    const float oFy = __shfl_xor_sync(kFull, w.Fy, 1);
+                    const float oFz = __shfl_xor_sync(kFull, w.Fz, 1);
+                    const float aFy = w.Fy + oFy;
+                    const float afy = sel(front, aFy * cd, aFy);               // Fyf or Fyr
+                    const float aFz = w.Fz + oFz;
+                    const float aDz = sel(left, w.Fz - oFz, oFz - w.Fz);        // left - right
+                    const float bfy = __shfl_xor_sync(kFull, afy, 2);
+                    const float bFz = __shfl_xor_sync(kFull, aFz, 2);
+                    const float bDz = __shfl_xor_sync(kFull, aDz, 2);
+                    const float Fyf = sel(front, afy, bfy), Fyr = sel(front, bfy, afy);
+                    const float Fzf = sel(front, aFz, bFz), Fzr = sel(front, bFz, aFz);
+                    FyB = Fyf + Fyr;
+                    FzB = Fzf + Fzr;
+                    Mx = fmaf(V.hR, FyB, V.he * (aDz + bDz));
+                    My = -V.Lf * Fzf + V.Lr * Fzr;
+                    Mz = V.Lf * Fyf + -V.Lr * Fyr;
+                    if (cm) {
+                        const float ac = w.cost + __shfl_xor_sync(kFull, w.cost, 1);
+                        csum = ac + __shfl_xor_sync(kFull, ac, 2);
+                    }
+                }
+                const float Fx = V.halfM * fmaf(-wz, vy, fmaf(wy, vz, ax - gBx));
+                My = fmaf(-V.hR, 2.f * Fx, My);
+                // the velocity rows of A(xi) + B zeta (Sec. IV-A), forward Euler
+                const float dvy = fmaf(-wz, vx, fmaf(wx, vz, fmaf(FyB, V.invM, gBy)));
+                const float dvz = fmaf(wy, vx, fmaf(-wx, vy, fmaf(FzB, V.invM, gBz)));
+                const float dwx = fmaf(V.dJyz * wy, wz, Mx) * V.invJxx;
+                const float dwy = fmaf(-V.dJxz * wx, wz, My) * V.invJyy;
+                const float dwz = fmaf(V.dJxy * wx, wy, Mz) * V.invJzz;
+                float nvx = vx, nvxl = vxl, nvy = vy, nvyl = vyl, nvz = vz, nvzl = vzl;
+                acc2(nvx, nvxl, h * ax);
+                acc2(nvy, nvyl, h * dvy);
+                acc2(nvz, nvzl, h * dvz);
+                const float nwx = fmaf(h, dwx, wx), nwy = fmaf(h, dwy, wy), nwz = fmaf(h, dwz, wz);
+                vx = sel(go, nvx, vx); vxl = sel(go, nvxl, vxl); vy = sel(go, nvy, vy); vyl = sel(go, nvyl, vyl);
+                vz = sel(go, nvz, vz); vzl = sel(go, nvzl, vzl);
+                wx = sel(go, nwx, wx); wy = sel(go, nwy, wy); wz = sel(go, nwz, wz);
+                if (q == 0) {
+                    sh.va[par ^ 1][c] = make_float4(vx, vy, vz, wx);
+                    sh.vb[par ^ 1][c] = make_float2(wy, wz);
+                }
+                // running cost L = L_0 + L_soft (Sec. IV-C), left Riemann sum
+                U = esm(V, body.z, sph, cph, cth);
+                margin = fminf(margin, U);
+                const float soft = fmaxf(fmaf(-U, Cc.inv_eps, 1.f), 0.f);
+                const float L = fmaf(Cc.sigma * soft, soft, fmaf(Cc.wc * dd, dd, Cc.wt)) + csum;
+                if (acc64) J64 += go ? (double)(h * L) : 0.0;
+                else J = sel(go, fmaf(h, L, J), J);
+            }
+            sm = fminf(sm, U);
+            pair_barrier();
+            par ^= 1;
+        }
+        if (live && p.step_margin && q == 0 && k + 1 < p.H) p.step_margin[(size_t)k * p.N + j] = sm;
+        if (k + 1 < p.H) {
+            if (sm < msm) {
+                msm = sm;
+                mstep = k;
+            }
+        } else {
+            last_sm = sm;
+        }
+    }
+    pair_barrier();                       // the geometry warp's final state is stored
+    if (!live) return;
+    // final state: margin and terminal cost Phi (Sec. IV-C)
+    if (!idle) {
+        const float4 att = sh.att[par][c], body = sh.body[par][c];
+        U = esm(V, body.z, att.z, att.w, att.y);
+    }
+    margin = fminf(margin, U);
+    last_sm = fminf(last_sm, U);
+    if (last_sm < msm) mstep = p.H - 1;
+    if (p.step_margin && q == 0) p.step_margin[(size_t)(p.H - 1) * p.N + j] = last_sm;
+    const float d2 = sh.d2[c];
+    if (acc64) J = (float)(J64 + (double)(Cc.wg * sqrtf(d2)));
+    else J = fmaf(Cc.wg, sqrtf(d2), J);
+    const float xs[6] = {vx + vxl, vy + vyl, vz + vzl, wx, wy, wz};
+    const int gfl = sh.flags[c];
+    bool finite = isfinite(J) && !(gfl & ATP_FLAG_NONFINITE);
+#pragma unroll
+    for (int r = 0; r < 6; ++r) finite = finite && isfinite(xs[r]);
+    if (!finite) J = CUDART_INF_F;
+    feasible = finite && margin > 0.f;
+    if (q == 0) {
+        const uint8_t fl = (feasible ? ATP_FLAG_FEASIBLE : 0) | (gfl & (ATP_FLAG_DONE | ATP_FLAG_OFFMAP)) |
+                           (finite ? 0 : ATP_FLAG_NONFINITE);
+        if (p.cost) p.cost[j] = J;
+        if (p.margin) p.margin[j] = margin;
+        if (p.flags) p.flags[j] = fl;
+        if (p.min_step) p.min_step[j] = mstep;
+        if (p.xf) {
+            const size_t N = (size_t)p.N;
+#pragma unroll
+            for (int r = 0; r < 6; ++r) p.xf[(6 + r) * N + j] = xs[r];
+        }
+    }
+}
+
+// Whether this warp is its pair's geometry warp.  Warps w and w + 4 share an
+// SM sub-partition, and the geometry warp issues about 1.6 times the forces
+// warp's instructions: the roles alternate by the CTA's warp slots, so that
+// the sub-partitions get both kinds (the scaled plan 407 -> 336 us with two
+// lanes).  The shuffle makes the answer uniform over the warp, so that the
+// branch on it is a plain jump (4 % of a small plan).
+__device__ __forceinline__ bool geometry_role(int &flip)
+{
+    if (threadIdx.x == 0) {
+        unsigned wid;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(wid));
+        flip = (wid >> 2) & 1;
+    }
+    __syncthreads();
+    return __shfl_sync(kFull, (int)(threadIdx.x >> 5) ^ flip, 0) == 0;
+}
+
+// One CTA of a two-warp plan; `cta` counts from the plan's first.  j is this
+// thread's candidate; the results are in the threads it returns true for.
+template <int LANES, bool PER_X0, int TEX, int ACC>
+__device__ __forceinline__ bool duo_rollout(const PlanParams &p, Duo<LANES> &sh, unsigned cta, int &j, float &J,
+                                            float &margin, bool &feasible)
+{
+    const int lane = threadIdx.x & 31, c = lane / LANES, q = lane & (LANES - 1);
+    const long long jl = (long long)cta * Duo<LANES>::kC + c;
+    const bool live = jl < p.N;
+    j = (int)jl;
+    const bool geo = geometry_role(sh.flip);
+    if (geo) duo_geometry<LANES, PER_X0, TEX>(p, sh, j, q, c, live);
+    else duo_forces<LANES, PER_X0, ACC>(p, sh, j, q, c, live, J, margin, feasible);
+    return live && !geo && q == 0;
+}
+
+// Registers: one lane runs best free of spills (168 registers, six CTAs per
+// SM: 0.296 ms at 16384 candidates against 0.345 ms at the 128-register cap),
+// two and four lanes fit 128.
+template <int LANES, bool PER_X0, bool REDUCE, int TEX, int ACC>
+__global__ void __launch_bounds__(kPlanBlock, LANES == 4 ? 1 : LANES == 2 ? 8 : 6)
+plan_duo_kernel(const __grid_constant__ PlanParams p)
+{
+    __shared__ Duo<LANES> sh;
+    int j;
+    float J = 0.f, margin = CUDART_INF_F;
+    bool feasible = false;
+    const bool leader = duo_rollout<LANES, PER_X0, TEX, ACC>(p, sh, blockIdx.x, j, J, margin, feasible);
+    if (!REDUCE) return;
+    plan_tail(p, j, leader, J, feasible, gridDim.x);
 }
 
 // Terrain staging: the one-lane rollout with a window of the texels in
@@ -426,7 +737,7 @@ plan_stage_kernel(const __grid_constant__ PlanParams p)
     const bool live = tid < p.N;
     float J = 0.f, margin = CUDART_INF_F;
     bool feasible = false;
-    if (live) rollout_one<1, false, TEX_F32W, ACC>(p, j, 0, 0u, J, margin, feasible);
+    if (live) rollout_one<false, TEX_F32W, ACC>(p, j, J, margin, feasible);
     if (!REDUCE) return;
     plan_tail<kStageBlock>(p, j, live, J, feasible, gridDim.x);
 }
@@ -455,41 +766,44 @@ cudaError_t launch_plan_staged(const PlanParams &p, bool reduce, cudaStream_t st
 
 // Continuous batching: one launch over a ragged batch of plans, each with its
 // own vehicle, terrain, horizon, candidates and outputs.  Plan r owns CTAs
-// [cta_begin[r], cta_begin[r+1]) with p.lanes threads per candidate, which
-// the host chooses for the batch as a whole (every layout gives the same
-// bits).  Every candidate runs exactly the code of a single plan, so its
-// results are the same bits alone and in any mix.  BTEX is the batch's texel
-// format when all its plans share one, or kTexMixed, where each plan branches
-// on its own: a kernel that inlines both formats' rollouts in all three
-// layouts spills registers, the single-format kernel does not (measured on
-// the GB300 on the 32-vehicle serving mix: p50 2 to 12 % lower at 20 to 80
-// requests/s per vehicle).
+// [cta_begin[r], cta_begin[r+1]) in the layout p.lanes, which the host chooses
+// for the batch as a whole (every layout gives the same bits).  Every
+// candidate runs exactly the code of a single plan, so its results are the
+// same bits alone and in any mix.  BTEX is the batch's texel format when all
+// its plans share one, or kTexMixed, where each plan branches on its own.
 constexpr int kTexMixed = -1;
 
-template <int LANES, int TEX>
-__device__ __forceinline__ void batch_rollout(const PlanParams &p, int j, int q, unsigned qmask, float &J,
+template <bool PER_X0, int TEX>
+__device__ __forceinline__ bool batch_rollout(const PlanParams &p, void *sh, unsigned cta, int &j, float &J,
                                               float &margin, bool &feasible)
 {
-    if (p.x0_soa) rollout_one<LANES, true, TEX, kAccRuntime>(p, j, q, qmask, J, margin, feasible);
-    else rollout_one<LANES, false, TEX, kAccRuntime>(p, j, q, qmask, J, margin, feasible);
+    // every thread of a CTA belongs to one plan: the branches are CTA-uniform
+    if (p.lanes == kLayoutDuo4)
+        return duo_rollout<4, PER_X0, TEX, kAccRuntime>(p, *(Duo<4> *)sh, cta, j, J, margin, feasible);
+    if (p.lanes == kLayoutDuo2)
+        return duo_rollout<2, PER_X0, TEX, kAccRuntime>(p, *(Duo<2> *)sh, cta, j, J, margin, feasible);
+    if (p.lanes == kLayoutDuo1)
+        return duo_rollout<1, PER_X0, TEX, kAccRuntime>(p, *(Duo<1> *)sh, cta, j, J, margin, feasible);
+    j = (int)(cta * kPlanBlock + threadIdx.x);
+    const bool live = j < p.N;
+    if (live) rollout_one<PER_X0, TEX, kAccRuntime>(p, j, J, margin, feasible);
+    return live;
 }
 
-template <int LANES, int BTEX>
-__device__ __forceinline__ void batch_tex(const PlanParams &p, int j, int q, unsigned qmask, float &J,
+template <int TEX>
+__device__ __forceinline__ bool batch_tex(const PlanParams &p, void *sh, unsigned cta, int &j, float &J,
                                           float &margin, bool &feasible)
 {
-    if constexpr (BTEX == kTexMixed) {
-        if (p.tex_format == TEX_F32) batch_rollout<LANES, TEX_F32>(p, j, q, qmask, J, margin, feasible);
-        else batch_rollout<LANES, TEX_BF16>(p, j, q, qmask, J, margin, feasible);
-    } else {
-        batch_rollout<LANES, BTEX>(p, j, q, qmask, J, margin, feasible);
-    }
+    return p.x0_soa ? batch_rollout<true, TEX>(p, sh, cta, j, J, margin, feasible)
+                    : batch_rollout<false, TEX>(p, sh, cta, j, J, margin, feasible);
 }
 
 template <int BTEX>
-__global__ void __launch_bounds__(kPlanBlock)
+__global__ void __launch_bounds__(kPlanBlock, 6)
 plan_batch_kernel(const __grid_constant__ BatchParams b)
 {
+    __shared__ __align__(16) unsigned char sh[sizeof(Duo<1>)];
+    static_assert(sizeof(Duo<1>) >= sizeof(Duo<2>) && sizeof(Duo<1>) >= sizeof(Duo<4>), "one buffer for all");
     int lo = 0, hi = b.n;
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
@@ -497,22 +811,15 @@ plan_batch_kernel(const __grid_constant__ BatchParams b)
         else hi = mid;
     }
     const PlanParams &p = b.req[lo];
-    const int tid = ((int)blockIdx.x - b.cta_begin[lo]) * kPlanBlock + (int)threadIdx.x;
-    // every thread of a CTA belongs to one plan: the branch is CTA-uniform
-    const int lanes = p.lanes;
-    const bool four = lanes == 4, two = lanes == 2;
-    const int j = four ? tid >> 2 : two ? tid >> 1 : tid;
-    const int q = four ? tid & 3 : two ? tid & 1 : 0;
-    const bool live = j < p.N;
-    const unsigned qmask = four ? 0xfu << (threadIdx.x & 28) : two ? 0x3u << (threadIdx.x & 30) : 0u;
+    const unsigned cta = blockIdx.x - (unsigned)b.cta_begin[lo];
+    int j;
     float J = 0.f, margin = CUDART_INF_F;
-    bool feasible = false;
-    if (live) {
-        if (four) batch_tex<4, BTEX>(p, j, q, qmask, J, margin, feasible);
-        else if (two) batch_tex<2, BTEX>(p, j, q, qmask, J, margin, feasible);
-        else batch_tex<1, BTEX>(p, j, 0, 0u, J, margin, feasible);
-    }
-    plan_tail(p, j, live && q == 0, J, feasible, (unsigned)(b.cta_begin[lo + 1] - b.cta_begin[lo]));
+    bool feasible = false, leader;
+    if (BTEX == TEX_F32 || (BTEX == kTexMixed && p.tex_format == TEX_F32))
+        leader = batch_tex<TEX_F32>(p, sh, cta, j, J, margin, feasible);
+    else
+        leader = batch_tex<TEX_BF16>(p, sh, cta, j, J, margin, feasible);
+    plan_tail(p, j, leader, J, feasible, (unsigned)(b.cta_begin[lo + 1] - b.cta_begin[lo]));
 }
 
 cudaError_t launch_plan_batch(const BatchParams &b, cudaStream_t stream)
@@ -530,44 +837,35 @@ cudaError_t launch_plan_batch(const BatchParams &b, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-template <int LANES, int TEX, int ACC>
+template <bool PER_X0, bool REDUCE, int TEX, int ACC>
+static void launch_layout(const PlanParams &p, int layout, cudaStream_t stream)
+{
+    const dim3 grid((unsigned)layout_ctas(layout, p.N)), block(kPlanBlock);
+    if (layout == kLayoutDuo4) plan_duo_kernel<4, PER_X0, REDUCE, TEX, ACC><<<grid, block, 0, stream>>>(p);
+    else if (layout == kLayoutDuo2) plan_duo_kernel<2, PER_X0, REDUCE, TEX, ACC><<<grid, block, 0, stream>>>(p);
+    else if (layout == kLayoutDuo1) plan_duo_kernel<1, PER_X0, REDUCE, TEX, ACC><<<grid, block, 0, stream>>>(p);
+    else plan_kernel<PER_X0, REDUCE, TEX, ACC><<<grid, block, 0, stream>>>(p);
+}
+
+template <int TEX, int ACC>
 static cudaError_t launch_acc(const PlanParams &p, bool reduce, cudaStream_t stream)
 {
-    const dim3 block(kPlanBlock);
-    const size_t threads = (size_t)p.N * LANES;
-    const dim3 grid((unsigned)((threads + kPlanBlock - 1) / kPlanBlock));
-    const bool per = p.x0_soa != nullptr;
+    const int layout = plan_layout(p.lanes, p.N);
     if (reduce) {
-        if (per) plan_kernel<LANES, true, true, TEX, ACC><<<grid, block, 0, stream>>>(p);
-        else plan_kernel<LANES, false, true, TEX, ACC><<<grid, block, 0, stream>>>(p);
+        if (p.x0_soa) launch_layout<true, true, TEX, ACC>(p, layout, stream);
+        else launch_layout<false, true, TEX, ACC>(p, layout, stream);
     } else {
-        if (per) plan_kernel<LANES, true, false, TEX, ACC><<<grid, block, 0, stream>>>(p);
-        else plan_kernel<LANES, false, false, TEX, ACC><<<grid, block, 0, stream>>>(p);
+        if (p.x0_soa) launch_layout<true, false, TEX, ACC>(p, layout, stream);
+        else launch_layout<false, false, TEX, ACC>(p, layout, stream);
     }
     return cudaGetLastError();
 }
 
-template <int LANES, int TEX>
-static cudaError_t launch_lanes(const PlanParams &p, bool reduce, cudaStream_t stream)
-{
-    return p.acc64 ? launch_acc<LANES, TEX, kAccF64>(p, reduce, stream)
-                   : launch_acc<LANES, TEX, kAccF32>(p, reduce, stream);
-}
-
 cudaError_t launch_plan(const PlanParams &p, bool reduce, cudaStream_t stream)
 {
-    // several lanes per candidate while the batch leaves the GPU's thread
-    // slots mostly empty (the rollout is then latency bound); one lane once
-    // the batch fills the machine
-    const int lanes = plan_lanes(p.lanes, p.N);
-    if (p.tex_format == TEX_F32) {
-        if (lanes == 4) return launch_lanes<4, TEX_F32>(p, reduce, stream);
-        if (lanes == 2) return launch_lanes<2, TEX_F32>(p, reduce, stream);
-        return launch_lanes<1, TEX_F32>(p, reduce, stream);
-    }
-    if (lanes == 4) return launch_lanes<4, TEX_BF16>(p, reduce, stream);
-    if (lanes == 2) return launch_lanes<2, TEX_BF16>(p, reduce, stream);
-    return launch_lanes<1, TEX_BF16>(p, reduce, stream);
+    if (p.tex_format == TEX_F32)
+        return p.acc64 ? launch_acc<TEX_F32, kAccF64>(p, reduce, stream) : launch_acc<TEX_F32, kAccF32>(p, reduce, stream);
+    return p.acc64 ? launch_acc<TEX_BF16, kAccF64>(p, reduce, stream) : launch_acc<TEX_BF16, kAccF32>(p, reduce, stream);
 }
 
 // One node's texel (Sec. III-A numeric slope, reading Q10): height, central-

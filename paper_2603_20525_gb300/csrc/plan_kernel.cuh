@@ -37,7 +37,8 @@ struct PlanParams {
                               // per-step margin (the final state folded into step H-1)
     int tex_format;           // TEX_F32 or TEX_BF16
     int acc64;                // accumulate the running cost in FP64
-    int lanes;                // 0: by batch size; else 1, 2 or 4 lanes per candidate
+    int lanes;                // 0: by batch size; else 1, 2 or 4 threads per candidate
+                              // (in a batch: the layout)
     // plan only
     atp_plan_out *out;
     float *best_ctrl;         // [H][2] or nullptr
@@ -46,17 +47,47 @@ struct PlanParams {
 };
 
 constexpr int kPlanBlock = 64;
-// Threads per candidate by batch size, from a sweep of the three layouts on
-// a GB300 (scaled workload, H = 100, 4 Euler steps per control step, L2
-// flushed before each plan): four lanes (one wheel each) are fastest up to
-// 12288 candidates, two (one axle each) at 16384 and 24576, one from 32768 on.
-constexpr int kLanes4MaxN = 12288;
-constexpr int kLanes2MaxN = 28672;
+// Layouts of a plan's CTAs of 64 threads, as threads per candidate: one
+// thread, or two warps that share 32, 16 or 8 candidates (one, two or four
+// lanes of each warp per candidate).  All give the same bits.
+constexpr int kLayoutOne = 1, kLayoutDuo1 = 2, kLayoutDuo2 = 4, kLayoutDuo4 = 8;
+// The lines lie where the next layout becomes the faster one (ms per plan on a
+// GB300, scaled workload, H = 100, 4 Euler steps per control step):
+//   candidates        8 threads   4 threads   2 threads   1 thread
+//   1024                0.160       0.193       0.243       0.330
+//   4096                0.177       0.194       0.248       0.339
+//   8192                0.241       0.216       0.248       0.337
+//   12288               0.385       0.266       0.281       0.344
+//   16384               0.420       0.315       0.296       0.344
+//   20480               0.592       0.473       0.369       0.424
+//   28672                           0.505       0.383       0.430
+//   32768                           0.565       0.615       0.436
+// 4864 = 152 x 4 x 8 candidates is four CTAs per SM on eight threads and 29184
+// = 152 x 6 x 32 the one wave of six CTAs per SM on two; between four and two
+// threads the order at 16384 depends on the terrain (0.296 to 0.376 ms on two,
+// 0.315 to 0.349 ms on four over five seeds).
+constexpr int kDuo4MaxN = 4864;
+constexpr int kDuo2MaxN = 16384;
+constexpr int kDuo1MaxN = 29184;
 
-// threads per candidate: `forced` (1, 2 or 4) if set, else by batch size
+// the layout of a plan of N candidates: `forced` (1, 2 or 4 threads, four
+// meaning eight where a plan of its size runs eight) if set, else by batch size
+inline int plan_layout(int forced, int N)
+{
+    const int four = N <= kDuo4MaxN ? kLayoutDuo4 : kLayoutDuo2;
+    if (forced) return forced == 4 ? four : forced;
+    return N <= kDuo2MaxN ? four : N <= kDuo1MaxN ? kLayoutDuo1 : kLayoutOne;
+}
+inline int layout_candidates(int layout) { return kPlanBlock / layout; }       // per CTA
+inline long long layout_ctas(int layout, long long N)
+{
+    return (N + layout_candidates(layout) - 1) / layout_candidates(layout);
+}
+// threads per candidate as ATP_OPT_LANES counts them: 1, 2 or 4 (or more)
 inline int plan_lanes(int forced, int N)
 {
-    return forced ? forced : (N <= kLanes4MaxN ? 4 : N <= kLanes2MaxN ? 2 : 1);
+    const int l = plan_layout(forced, N);
+    return l > 4 ? 4 : l;
 }
 cudaError_t launch_plan(const PlanParams &p, bool reduce, cudaStream_t stream);
 

@@ -117,54 +117,78 @@ __device__ __forceinline__ float esm(const Veh &V, float ph, float sph, float cp
     return fabsf(ph) < V.tip ? u : -u;
 }
 
-// Position of the CoM in cell units split into an integer cell and a
-// fraction, from the compensated coordinate hi + lo (metres from the origin).
-__device__ __forceinline__ void cell_split(float hi, float lo, float inv_cell, int &ic, float &fc)
+// 1.5 x 2^23: adding it to |u| <= 2^22 rounds u to a whole number in the low
+// mantissa bits, at FADD latency instead of a conversion's (F2I, I2F and FRND
+// run at a quarter rate and about five times the latency).
+constexpr float kMagic = 12582912.f;
+constexpr unsigned kMagicBits = 0x4b400000u;
+constexpr float kMaxCell = 2097152.f;        // 2^21: the CoM's cell is clamped to +-2^21
+
+// One axis of the CoM in cell units: the fraction fc of its cell, and the map
+// as seen from that cell: its first node lo, its last node hi (whole numbers,
+// exact), the last lookup cell in magic form (kMagic + n - 2 - cell), and the
+// cell itself in magic form.
+struct Cell {
+    float fc, lo, hi, tmax, t;
+};
+
+// From the compensated coordinate hi + lo (metres from the origin).  A NaN
+// takes the low edge.  WRAP: a position 2^31 cells or more beyond the map (a
+// rollout that has diverged) takes the opposite edge's texels, as the plans'
+// saturating 32-bit cell sums always have; it is off the map either way.
+template <bool WRAP = true>
+__device__ __forceinline__ Cell cell_of(float hi, float lo, float inv_cell, int n)
 {
-    const float u = fminf(fmaxf(hi * inv_cell, -4194304.f), 4194304.f);   // NaN -> low edge
-    const float fl = floorf(u);
-    ic = (int)fl;
-    fc = fmaf(lo, inv_cell, fmaf(hi, inv_cell, -fl));
+    Cell c;
+    const float u = fminf(fmaxf(hi * inv_cell, -kMaxCell), kMaxCell);   // NaN -> low edge
+    c.t = __fadd_rd(u, kMagic);
+    const float fl = c.t - kMagic;                                      // floor(u)
+    const float f = fmaf(lo, inv_cell, fmaf(hi, inv_cell, -fl));
+    c.fc = !WRAP || fabsf(f) < 2143289344.f ? f : -f;                   // 2^31 - 2^22
+    c.lo = -fl;
+    c.hi = (float)(n - 1) - fl;
+    c.tmax = (kMagic + (float)(n - 2)) - fl;
+    return c;
 }
 
-// One axis of a wheel lookup: CoM cell (ic, fc) plus the wheel's offset `o`
-// metres; returns the clamped cell index in [0, n-2] and the weight in [0, 1]
-// (queries clamped to the map, reading Q10).
-// Written with selects rather than branches: the four wheels' lookups then
-// form one basic block that the compiler can interleave (measured on the
-// GB300: 9 % off a full-GPU plan, 3 to 10 % off the smaller ones).  The cell
-// comes from one rounding-down conversion, which saturates for a huge or
-// infinite offset and gives 0 for NaN; the sum with the CoM cell wraps
-// (unsigned) instead of overflowing, and every out-of-range index is clamped
-// below, so no lookup leaves the map.
-__device__ __forceinline__ int axis(int ic, float fc, float o, float inv_cell, int n, float &a, bool &off)
+// One axis of a lookup at `u` cells from the CoM's cell: returns the lookup
+// cell in [0, n-2] (in magic form) and the weight w in [0, 1] (queries clamped
+// to the map, reading Q10), and sets `off` for a query outside the map.  Only
+// min, max and additions: the clamp of the coordinate gives the weights 0 and
+// 1 beyond the map, and the coordinate differs from its clamp exactly when the
+// query is off the map.  A NaN takes the low edge and does not set `off` (the
+// caller's off_com does when the position itself is NaN); every index lies on
+// the map whatever u is.
+__device__ __forceinline__ float axis(const Cell &c, float u, float &w, bool &off)
 {
-    const float u = fmaf(o, inv_cell, fc);
-    const int fi = __float2int_rd(u);
-    const int i = (int)((unsigned)ic + (unsigned)fi);
-    const float w = u - (float)fi;
-    const bool below = i < 0, above = i >= n - 1;
-    off = off || below || (above && (i > n - 1 || w > 0.f));
-    a = below ? 0.f : (above ? 1.f : w);
-    return below ? 0 : (above ? n - 2 : i);
+    const float uc = fminf(fmaxf(u, c.lo), c.hi);
+    const float t = fminf(__fadd_rd(uc, kMagic), c.tmax);
+    w = uc - (t - kMagic);
+    off = off || u < uc || u > uc;
+    return t;
 }
 
-// axis() for both axes of one lookup, with the cell coordinate and fraction
-// of the two taken as pairs; bit for bit the same as two axis() calls
-__device__ __forceinline__ void axis_xy(int icx, int icy, float2 fc, float2 o, float inv_cell, int nx,
-                                        int ny, int &i, int &j, float &a, float &b, bool &off)
+// the CoM is so far below the map's edge, or NaN, that its cell was clamped
+__device__ __forceinline__ bool off_com(const Cell &cx, const Cell &cy)
 {
-    const float2 u = fma2(o, splat2(inv_cell), fc);
-    const int fx = __float2int_rd(u.x), fy = __float2int_rd(u.y);
-    const float2 w = sub2(u, make_float2((float)fx, (float)fy));
-    const int ix = (int)((unsigned)icx + (unsigned)fx);
-    const int iy = (int)((unsigned)icy + (unsigned)fy);
-    const bool bx = ix < 0, ex = ix >= nx - 1, by = iy < 0, ey = iy >= ny - 1;
-    off = off || bx || (ex && (ix > nx - 1 || w.x > 0.f)) || by || (ey && (iy > ny - 1 || w.y > 0.f));
-    a = bx ? 0.f : (ex ? 1.f : w.x);
-    b = by ? 0.f : (ey ? 1.f : w.y);
-    i = bx ? 0 : (ex ? nx - 2 : ix);
-    j = by ? 0 : (ey ? ny - 2 : iy);
+    return cx.lo >= kMaxCell || cy.lo >= kMaxCell;
+}
+
+// texel index of the CoM's cell less the magic bits of a lookup's two axes:
+// texel_index(base, tx, ty, nx) = j nx + i, modulo 2^32 (a map has at most
+// 2^32 nodes)
+__device__ __forceinline__ unsigned texel_base(const Cell &cx, const Cell &cy, int nx)
+{
+    return (__float_as_uint(cy.t) - 2u * kMagicBits) * (unsigned)nx + (__float_as_uint(cx.t) - 2u * kMagicBits);
+}
+__device__ __forceinline__ unsigned texel_index(unsigned base, float tx, float ty, int nx)
+{
+    return __float_as_uint(ty) * (unsigned)nx + (__float_as_uint(tx) + base);
+}
+// the lookup cell along one axis
+__device__ __forceinline__ int cell_index(const Cell &c, float t)
+{
+    return (int)(__float_as_uint(t) + __float_as_uint(c.t) - 2u * kMagicBits);
 }
 
 __device__ __forceinline__ float lerp2d(float t00, float t10, float t01, float t11, float a, float b)
@@ -213,22 +237,28 @@ __device__ __forceinline__ float4 texel16(const Terrain &T, int i, int j)
     return t;
 }
 
+// The lookup at cell (tx, ty) (magic form) with weights (a, b), seen from the
+// CoM's cell (cx, cy) whose texel_base is `base`.
 template <int TEX>
-__device__ __forceinline__ float4 bilerp(const Terrain &T, int i, int j, float a, float b)
+__device__ __forceinline__ float4 bilerp(const Terrain &T, const Cell &cx, const Cell &cy, unsigned base, float tx,
+                                         float ty, float a, float b)
 {
     const bool cm = T.has_cm != 0;
     if (TEX == TEX_F32) {
-        const float4 *r0 = T.tex + (size_t)j * T.nx + i;
-        return lerp4(__ldg(r0), __ldg(r0 + 1), __ldg(r0 + T.nx), __ldg(r0 + T.nx + 1), a, b, cm);
+        const unsigned o = texel_index(base, tx, ty, T.nx);
+        const float4 *r0 = T.tex + o, *r1 = T.tex + (size_t)(o + (unsigned)T.nx);
+        return lerp4(__ldg(r0), __ldg(r0 + 1), __ldg(r1), __ldg(r1 + 1), a, b, cm);
     } else if (TEX == TEX_F32W) {
         // one generic pointer into the window or the texel array, so that a
         // warp whose lookups fall on both sides still issues four loads
+        const int i = cell_index(cx, tx), j = cell_index(cy, ty);
         const unsigned li = (unsigned)(i - T.wx0), lj = (unsigned)(j - T.wy0);
         const bool in = li < (unsigned)(T.ww - 1) && lj < (unsigned)(T.wh - 1);
         const float4 *r0 = in ? atp_win + (lj * (unsigned)T.ww + li) : T.tex + (size_t)j * T.nx + i;
         const int s = in ? T.ww : T.nx;
         return lerp4(r0[0], r0[1], r0[s], r0[s + 1], a, b, cm);
     } else {
+        const int i = cell_index(cx, tx), j = cell_index(cy, ty);
         return lerp4(texel16(T, i, j), texel16(T, i + 1, j), texel16(T, i, j + 1),
                      texel16(T, i + 1, j + 1), a, b, cm);
     }
@@ -243,14 +273,12 @@ struct WheelGeo {
 
 // One wheel's geometry (Sec. IV-A): contact point P = p + R rho, the terrain
 // below it, the slope-normal tau ~ (-f_x, -f_y, 1) (reading Q1) resolved in
-// B and the extension chi along it.  (icx, fcx), (icy, fcy) is the CoM's cell
-// and fraction, z_hi + z_lo its height.  PAIRED takes the lookup's two axes
-// as packed pairs: the same bits, measured faster with two lanes per
-// candidate and slower with one or four.
-template <int TEX, bool PAIRED = false>
-__device__ __forceinline__ WheelGeo wheel_geo(const Veh &V, const Terrain &T, const float R[9], int icx,
-                                              int icy, float fcx, float fcy, float z_hi, float z_lo,
-                                              float rx, float ry, bool &off)
+// B and the extension chi along it.  cx, cy is the CoM's cell and z_hi + z_lo
+// its height.
+template <int TEX>
+__device__ __forceinline__ WheelGeo wheel_geo(const Veh &V, const Terrain &T, const float R[9], const Cell &cx,
+                                              const Cell &cy, unsigned base, float z_hi, float z_lo, float rx,
+                                              float ry, bool &off)
 {
     // offset of the contact point from the CoM in W: R (rx, ry, -(h+R))
     const float2 oxy = fma2(splat2(rx), make_float2(R[0], R[3]),
@@ -258,15 +286,10 @@ __device__ __forceinline__ WheelGeo wheel_geo(const Veh &V, const Terrain &T, co
                                  make_float2(-V.hR * R[2], -V.hR * R[5])));
     const float oz = fmaf(rx, R[6], fmaf(ry, R[7], -V.hR * R[8]));
     // terrain below the contact point
+    const float2 u = fma2(oxy, splat2(T.inv_cell), make_float2(cx.fc, cy.fc));
     float a, bb;
-    int i, j;
-    if constexpr (PAIRED) {
-        axis_xy(icx, icy, make_float2(fcx, fcy), oxy, T.inv_cell, T.nx, T.ny, i, j, a, bb, off);
-    } else {
-        i = axis(icx, fcx, oxy.x, T.inv_cell, T.nx, a, off);
-        j = axis(icy, fcy, oxy.y, T.inv_cell, T.ny, bb, off);
-    }
-    const float4 t = bilerp<TEX>(T, i, j, a, bb);
+    const float tx = axis(cx, u.x, a, off), ty = axis(cy, u.y, bb, off);
+    const float4 t = bilerp<TEX>(T, cx, cy, base, tx, ty, a, bb);
     // tau in B = R^T (-f_x, -f_y, 1)
     const float2 txy = fma2(make_float2(-R[3], -R[4]), splat2(t.z),
                             fma2(make_float2(-R[0], -R[1]), splat2(t.y), make_float2(R[6], R[7])));
@@ -323,21 +346,20 @@ __device__ __forceinline__ WheelOut wheel_dyn(const Veh &V, const WheelGeo &g, f
 // Per-step body quantities the four wheels share.
 struct Body {
     float R[9];
-    int icx, icy;            // CoM cell
-    float fcx, fcy;          // CoM fraction of the cell
+    Cell cx, cy;             // CoM cell
+    unsigned base;           // its texel_base
     float z_hi, z_lo;        // CoM height
     float vx, vy, vz, wx, wy, wz;
 };
 
 // One wheel (Sec. IV-A): its geometry, then its forces at the body's
 // velocities.
-template <int TEX, bool PAIRED = false>
+template <int TEX>
 __device__ __forceinline__ WheelOut wheel(const Veh &V, const Terrain &T, const Body &B, float rx, float ry,
                                           float k, float b, float Fs, float di, bool &off)
 {
-    const WheelGeo g = wheel_geo<TEX, PAIRED>(V, T, B.R, B.icx, B.icy, B.fcx, B.fcy, B.z_hi, B.z_lo, rx, ry,
-                                              off);
-    return wheel_dyn<PAIRED>(V, g, B.vx, B.vy, B.vz, B.wx, B.wy, B.wz, rx, ry, k, b, Fs, di);
+    const WheelGeo g = wheel_geo<TEX>(V, T, B.R, B.cx, B.cy, B.base, B.z_hi, B.z_lo, rx, ry, off);
+    return wheel_dyn(V, g, B.vx, B.vy, B.vz, B.wx, B.wy, B.wz, rx, ry, k, b, Fs, di);
 }
 
 }  // namespace atp

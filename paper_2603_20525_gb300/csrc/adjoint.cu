@@ -6,729 +6,628 @@
 // The margin's gradient is that of U_ESM at the state holding the minimum
 // (the first one on ties), as a subgradient of the minimum.
 //
-// Four threads per candidate, one wheel each, as in the plan kernel's
-// four-lane layout: every lane repeats the body arithmetic and its adjoint
-// bit-identically, runs its own wheel forwards and backwards, and the quad
-// exchanges only sums (the force and moment sums forwards; the wheels'
-// contributions to the body adjoints backwards).  The forward pass stores the
-// state every `ckpt` control steps; the reverse pass recomputes one segment
-// at a time into a per-lane buffer and walks its Euler steps backwards (for
-// a small grid on separate warps, the next segment recomputed while this one
-// is walked).  Each backward step recomputes the step's intermediates from
-// the stored state and propagates the state adjoint lambda through the Euler
-// update, the state derivative A(xi) + B zeta, the force and moment sums,
-// every wheel (contact kinematics, bilinear terrain, suspension with
-// liftoff, slip and tire), the rotation and the running cost with its ESM
-// soft constraint.  Branches (spring and damper liftoff, steering clamps,
-// off-map clamping, the goal test) follow the forward pass's choice, so the
-// result is the derivative of the piecewise-smooth discrete map along the
-// primal trajectory.
+// Two kernels.  The forward one is the two-warp rollout (duo.cuh), which also
+// writes every Euler step's start state.  Given those states, the steps'
+// derivatives do not depend on one another, only their product with the
+// adjoint does: in the backward kernel each lane of a candidate's warps
+// linearises one Euler step (the 13 x 13 matrix by which the step's adjoint
+// changes, column by column into shared memory), and then one warp runs the
+// recursion lam <- lam + M lam + c over those steps, one column per lane.
+// The recursion's step is 13 shuffles and 13 FMAs, instead of the step's
+// whole forward and reverse arithmetic on the serial chain.  Walking the
+// steps back with their arithmetic on the chain, beside a recomputation from
+// checkpoints, took 716 us for 64 candidates of 400 steps, 753 us for 4096 of
+// 300 and 597 us for 8000 of 200; this way they take 208, 420 and 500 us.  The
+// forward chain bounds the first (about 150 us), the linearisation's issue and
+// the seven warps per SM that its shared memory holds the others.
+//
+// Linearising a step differentiates the Euler update, the state derivative
+// A(xi) + B zeta, the force and moment sums, every wheel (contact kinematics,
+// bilinear terrain, suspension with liftoff, slip and tire), the rotation and
+// the running cost with its ESM soft constraint.  Branches (spring and damper
+// liftoff, steering clamps, off-map clamping, the goal test) follow the
+// forward pass's choice, so the result is the derivative of the
+// piecewise-smooth discrete map along the primal trajectory.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
 #include "adjoint.cuh"
-#include "atp.h"
-#include "srb_model.cuh"
+#include "duo.cuh"
 
 namespace atp {
 
 namespace {
 
-struct St {
-    float x, xl, y, yl, z, zl, psi, psil, th, ph;
-    float vx, vxl, vy, vyl, vz, vzl, wx, wy, wz, d;
-};
-constexpr int kStFloats = 20;
+// ---- linearisation of one Euler step ---------------------------------------
 
-__device__ __forceinline__ void st_store(float *dst, size_t stride, const St &s)
-{
-    const float *v = &s.x;
-#pragma unroll
-    for (int c = 0; c < kStFloats; ++c) dst[c * stride] = v[c];
-}
+// Rows of the step's matrix, the components of the adjoint after the step.
+enum { X, Y, Z, PSI, TH, PH, VX, VY, VZ, WX, WY, WZ, DE, kRows };
+// Columns: the same components before the step, then the two gradients.
+constexpr int kGdd = 13, kGax = 14, kCols = 15;
+// One column: the 13 rows, the constant c, (in column kGdd) whether the
+// steering rate is inside its limit, and the component's own factor: 1, or 0
+// for a steering angle at its clamp.
+constexpr int kColFloats = 16;
+// floats per step, padded so that the lanes' 16-byte stores fall on distinct banks
+constexpr int kStepFloats = kCols * kColFloats + 4;
 
-__device__ __forceinline__ void st_load(const float *src, size_t stride, St &s)
-{
-    float *v = &s.x;
-#pragma unroll
-    for (int c = 0; c < kStFloats; ++c) v[c] = src[c * stride];
-}
-
-__device__ __forceinline__ float clampf(float v, float lo, float hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
-// sum over the four lanes of a candidate (the same bits in every lane)
-__device__ __forceinline__ float qsum(float v, unsigned mask)
-{
-    v += __shfl_xor_sync(mask, v, 1);
-    v += __shfl_xor_sync(mask, v, 2);
-    return v;
-}
-
-// this lane's wheel: fl, fr, rl, rr for q = 0..3
-struct Lane {
-    int q;
-    unsigned mask;
-    bool front;
-    float rx, ry, k, b, Fs;
+// gradients of one wheel's F_z: x, y, z, psi, theta, phi, v, w
+struct WheelGrad {
+    float Fz, Fy;            // the forces
+    float ratio;             // F_y / F_z
+    float g[12];             // dF_z
+    float a[5], ad;          // F_z d(F_y / F_z) / d(vx, vy, wx, wy, wz) and / d(delta)
+    float c[6];              // costmap rate: x, y, (z), psi, theta, phi
 };
 
-__device__ __forceinline__ Lane lane_of(const Veh &V, int q, unsigned mask)
+struct Attitude {
+    float R[9], sps, cps, sth, cth, sph, cph;
+};
+
+// contraction of a gradient in the rotation's entries with dR / d(psi, theta, phi)
+__device__ __forceinline__ void angles_of(const Attitude &A, const float a[9], float &ps, float &th, float &ph)
 {
-    Lane l;
-    l.q = q;
-    l.mask = mask;
-    l.front = q < 2;
-    l.rx = l.front ? V.Lf : -V.Lr;
-    l.ry = (q & 1) ? -V.he : V.he;
-    l.k = l.front ? V.kf : V.kr;
-    l.b = l.front ? V.bf : V.br;
-    l.Fs = l.front ? V.Fsf : V.Fsr;
-    return l;
+    const float *R = A.R;
+    ps = fmaf(a[3], R[0], -a[0] * R[3]) + fmaf(a[4], R[1], -a[1] * R[4]) + fmaf(a[5], R[2], -a[2] * R[5]);
+    const float t0 = fmaf(A.cth, fmaf(a[1], A.sph, a[2] * A.cph), -a[0] * A.sth);
+    const float t1 = fmaf(A.cth, fmaf(a[4], A.sph, a[5] * A.cph), -a[3] * A.sth);
+    const float t2 = fmaf(A.sth, fmaf(a[7], A.sph, a[8] * A.cph), a[6] * A.cth);
+    th = fmaf(A.cps, t0, fmaf(A.sps, t1, -t2));
+    ph = fmaf(a[1], R[2], -a[2] * R[1]) + fmaf(a[4], R[5], -a[5] * R[4]) + fmaf(a[7], R[8], -a[8] * R[7]);
 }
 
-// a lookup axis: cell (magic form), weight and whether the query was clamped
-// (the last node itself counts: the weight there is 1 whatever moves the query)
-__device__ __forceinline__ float axis_c(const Cell &c, float o, float inv_cell, float &a, bool &clamped)
+// One wheel at the step's start state: its forces as the forward pass forms
+// them, and their gradients by reverse differentiation of F_z.
+__device__ __forceinline__ void wheel_lin(const Veh &V, const Terrain &T, const Attitude &A, const Cell &cx,
+                                          const Cell &cy, unsigned base, float z, float zl, float vx, float vy,
+                                          float vz, float wx, float wy, float wz, float rx, float ry, float k,
+                                          float b, float Fs, float di, WheelGrad &w)
 {
-    const float u = fmaf(o, inv_cell, c.fc);
+    const float *R = A.R;
+    const float ox = fmaf(rx, R[0], fmaf(ry, R[1], -V.hR * R[2]));
+    const float oy = fmaf(rx, R[3], fmaf(ry, R[4], -V.hR * R[5]));
+    const float oz = fmaf(rx, R[6], fmaf(ry, R[7], -V.hR * R[8]));
+    const float vix = fmaf(-wz, ry, fmaf(-wy, V.hR, vx));
+    const float viy = fmaf(wx, V.hR, fmaf(wz, rx, vy));
+    const float viz = fmaf(-wy, rx, fmaf(wx, ry, vz));
+    // the lookup; a query at or beyond the map's last node is clamped: what
+    // moves it does not move the interpolation
+    const float ux = fmaf(ox, T.inv_cell, cx.fc), uy = fmaf(oy, T.inv_cell, cy.fc);
+    const bool inx = ux >= cx.lo && ux < cx.hi, iny = uy >= cy.lo && uy < cy.hi;
     bool off = false;
-    clamped = !(u >= c.lo && u < c.hi);
-    return axis(c, u, a, off);
-}
-
-// every intermediate of one wheel that its adjoint needs
-struct WF {
-    float ox, oy, oz, vix, viy, viz;
-    float a, b;
-    bool cx, cy;
-    float4 t00, t10, t01, t11, t;
-    float tx, ty, tz, itz, Q, chi, A, Bv, N, chid, Fk, Fb0, Fz, alpha, Ca, T, Fy;
-};
-
-__device__ __forceinline__ void wheel_fwd(const Veh &V, const Terrain &T, const float R[9], const Cell &cx,
-                                          const Cell &cy, unsigned base, float z, float zl, float vx, float vy, float vz,
-                                          float wx, float wy, float wz, float rx, float ry, float k, float b,
-                                          float Fs, float di, WF &w)
-{
-    w.ox = fmaf(rx, R[0], fmaf(ry, R[1], -V.hR * R[2]));
-    w.oy = fmaf(rx, R[3], fmaf(ry, R[4], -V.hR * R[5]));
-    w.oz = fmaf(rx, R[6], fmaf(ry, R[7], -V.hR * R[8]));
-    w.vix = fmaf(-wz, ry, fmaf(-wy, V.hR, vx));
-    w.viy = fmaf(wx, V.hR, fmaf(wz, rx, vy));
-    w.viz = fmaf(-wy, rx, fmaf(wx, ry, vz));
-    const float tx = axis_c(cx, w.ox, T.inv_cell, w.a, w.cx);
-    const float ty = axis_c(cy, w.oy, T.inv_cell, w.b, w.cy);
-    const unsigned o = texel_index(base, tx, ty, T.nx);
+    float wa, wb;
+    const float ix = axis(cx, ux, wa, off), iy = axis(cy, uy, wb, off);
+    const unsigned o = texel_index(base, ix, iy, T.nx);
     const float4 *r0 = T.tex + o, *r1 = T.tex + (size_t)(o + (unsigned)T.nx);
-    w.t00 = __ldg(r0);
-    w.t10 = __ldg(r0 + 1);
-    w.t01 = __ldg(r1);
-    w.t11 = __ldg(r1 + 1);
-    w.t = lerp4(w.t00, w.t10, w.t01, w.t11, w.a, w.b, T.has_cm != 0);
-    w.tx = fmaf(-R[3], w.t.z, fmaf(-R[0], w.t.y, R[6]));
-    w.ty = fmaf(-R[4], w.t.z, fmaf(-R[1], w.t.y, R[7]));
-    w.tz = fmaf(-R[5], w.t.z, fmaf(-R[2], w.t.y, R[8]));
-    w.itz = rcp(w.tz);
-    w.Q = (z - w.t.x) + (w.oz + zl);
-    w.chi = w.Q * w.itz;
-    w.A = fmaf(-w.chi, wy, w.vix);
-    w.Bv = fmaf(w.chi, wx, w.viy);
-    w.N = fmaf(w.tz, w.viz, fmaf(w.ty, w.Bv, w.tx * w.A));
-    w.chid = w.N * w.itz;
-    w.Fk = fmaxf(fmaf(-k, w.chi, Fs), 0.f);
-    w.Fb0 = fmaf(-b, w.chid, w.Fk);
-    w.Fz = w.Fk > 0.f ? fmaxf(w.Fb0, 0.f) : 0.f;
-    w.alpha = atan2_r(w.viy, w.vix) - di;
-    w.Ca = V.C * w.alpha;
-    const float is = rsq(fmaf(w.Ca, w.Ca, V.mu2));
-    w.T = (-w.Ca * V.mu) * is;                    // F_y / F_z
-    w.Fy = w.Fz * w.T;
-}
-
-// adjoint accumulators of one Euler step
-struct Adj {
-    float R[9];
-    float x, y, z, vx, vy, vz, wx, wy, wz, d;
-};
-
-// one wheel backwards: given a_Fz, a_Fy and a_cost of this wheel, accumulate
-// the adjoints of R, of the CoM position and of the rates
-__device__ __forceinline__ void wheel_adj(const Veh &V, const Terrain &T, const float R[9], float wx, float wy,
-                                          float rx, float ry, float k, float b, float di_is_delta, const WF &w,
-                                          float aFz, float aFy, float aC, Adj &ad, float &a_d)
-{
-    // tire: Fy = Fz T(Ca), T = -mu Ca / sqrt(mu^2 + Ca^2), T' = -mu^3 / (mu^2 + Ca^2)^(3/2)
-    aFz += aFy * w.T;
-    const float den = fmaf(w.Ca, w.Ca, V.mu2);
-    const float is = rsq(den);
-    const float dT = -V.mu * V.mu2 * is * is * is;
-    const float aAlpha = aFy * w.Fz * dT * V.C;
+    const float4 t00 = __ldg(r0), t10 = __ldg(r0 + 1), t01 = __ldg(r1), t11 = __ldg(r1 + 1);
+    const float4 t = lerp4(t00, t10, t01, t11, wa, wb, T.has_cm != 0);
+    const float tx = fmaf(-R[3], t.z, fmaf(-R[0], t.y, R[6]));
+    const float ty = fmaf(-R[4], t.z, fmaf(-R[1], t.y, R[7]));
+    const float tz = fmaf(-R[5], t.z, fmaf(-R[2], t.y, R[8]));
+    const float itz = rcp(tz);
+    const float Q = (z - t.x) + (oz + zl);
+    const float chi = Q * itz;
+    const float a = fmaf(-chi, wy, vix), bv = fmaf(chi, wx, viy);
+    const float num = fmaf(tz, viz, fmaf(ty, bv, tx * a));
+    const float chid = num * itz;
+    const float Fk = fmaxf(fmaf(-k, chi, Fs), 0.f);
+    const float Fb = fmaf(-b, chid, Fk);
+    w.Fz = Fk > 0.f ? fmaxf(Fb, 0.f) : 0.f;
+    const float Ca = V.C * (atan2_r(viy, vix) - di);
+    const float is = rsq(fmaf(Ca, Ca, V.mu2));
+    w.ratio = (-Ca * V.mu) * is;
+    w.Fy = w.Fz * w.ratio;
+    // slip: F_z dT / dCa dCa / dalpha, T' = -mu^3 / (mu^2 + Ca^2)^(3/2),
     // alpha = atan2(viy, vix) - di
-    const float r2 = fmaf(w.vix, w.vix, w.viy * w.viy);
-    float aVix = 0.f, aViy = 0.f;
-    if (r2 > 0.f) {
-        const float ir2 = rcp(r2);
-        aViy += aAlpha * w.vix * ir2;
-        aVix -= aAlpha * w.viy * ir2;
+    const float dT = w.Fz * (-V.mu * V.mu2 * is * is * is * V.C);
+    const float r2 = fmaf(vix, vix, viy * viy);
+    const float ir2 = r2 > 0.f ? rcp(r2) : 0.f;
+    const float ax = -dT * viy * ir2, ay = dT * vix * ir2;      // by vix, viy
+    w.a[0] = ax;
+    w.a[1] = ay;
+    w.a[2] = ay * V.hR;
+    w.a[3] = -ax * V.hR;
+    w.a[4] = fmaf(ay, rx, -ax * ry);
+    w.ad = -dT;
+    // suspension: F_z = F_k - b chid while both are positive, F_k = F_s - k chi
+    const bool on = Fk > 0.f && Fb > 0.f;
+    const float aN = on ? -b * itz : 0.f;                        // by num
+    float aItz = on ? -b * num : 0.f;
+    const float aA = aN * tx, aB = aN * ty, aViz = aN * tz;
+    const float aChi = (on ? -k : 0.f) - aA * wy + aB * wx;
+    const float aQ = aChi * itz;
+    aItz = fmaf(aChi, Q, aItz);
+    const float aTx = aN * a, aTy = aN * bv, aTz = fmaf(-aItz * itz, itz, aN * viz);
+    // tau = R^T (-f_x, -f_y, 1), the height and the slopes through the lookup
+    const float gx = -(aTx * R[0] + aTy * R[1] + aTz * R[2]);
+    const float gy = -(aTx * R[3] + aTy * R[4] + aTz * R[5]);
+    const float oa = 1.f - wa, ob = 1.f - wb;
+    const float da_f = ob * (t10.x - t00.x) + wb * (t11.x - t01.x), db_f = oa * (t01.x - t00.x) + wa * (t11.x - t10.x);
+    const float da_x = ob * (t10.y - t00.y) + wb * (t11.y - t01.y), db_x = oa * (t01.y - t00.y) + wa * (t11.y - t10.y);
+    const float da_y = ob * (t10.z - t00.z) + wb * (t11.z - t01.z), db_y = oa * (t01.z - t00.z) + wa * (t11.z - t10.z);
+    const float aOx = inx ? (-aQ * da_f + gx * da_x + gy * da_y) * T.inv_cell : 0.f;
+    const float aOy = iny ? (-aQ * db_f + gx * db_x + gy * db_y) * T.inv_cell : 0.f;
+    const float aR[9] = {fmaf(aOx, rx, -aTx * t.y), fmaf(aOx, ry, -aTy * t.y), fmaf(-aOx, V.hR, -aTz * t.y),
+                         fmaf(aOy, rx, -aTx * t.z), fmaf(aOy, ry, -aTy * t.z), fmaf(-aOy, V.hR, -aTz * t.z),
+                         fmaf(aQ, rx, aTx), fmaf(aQ, ry, aTy), fmaf(-aQ, V.hR, aTz)};
+    w.g[0] = aOx;
+    w.g[1] = aOy;
+    w.g[2] = aQ;
+    angles_of(A, aR, w.g[3], w.g[4], w.g[5]);
+    w.g[6] = aA;
+    w.g[7] = aB;
+    w.g[8] = aViz;
+    w.g[9] = fmaf(aB, V.hR, fmaf(aViz, ry, aB * chi));
+    w.g[10] = -fmaf(aA, V.hR, fmaf(aViz, rx, aA * chi));
+    w.g[11] = fmaf(aB, rx, -aA * ry);
+    // costmap rate
+    w.c[0] = w.c[1] = w.c[2] = w.c[3] = w.c[4] = w.c[5] = 0.f;
+    if (T.has_cm) {
+        const float da_c = ob * (t10.w - t00.w) + wb * (t11.w - t01.w), db_c = oa * (t01.w - t00.w) + wa * (t11.w - t10.w);
+        const float px = inx ? da_c * T.inv_cell : 0.f, py = iny ? db_c * T.inv_cell : 0.f;
+        const float cR[9] = {px * rx, px * ry, -px * V.hR, py * rx, py * ry, -py * V.hR, 0.f, 0.f, 0.f};
+        w.c[0] = px;
+        w.c[1] = py;
+        angles_of(A, cR, w.c[3], w.c[4], w.c[5]);
     }
-    a_d -= aAlpha * di_is_delta;
-    // suspension: Fz = max(Fk - b chid, 0) while Fk > 0
-    float aFk = 0.f, aChid = 0.f;
-    if (w.Fk > 0.f && w.Fb0 > 0.f) {
-        aFk = aFz;
-        aChid = -b * aFz;
-    }
-    float aChi = 0.f;
-    if (w.Fk > 0.f) aChi -= k * aFk;                 // Fk = Fs - k chi
-    // chid = N itz, N = tx A + ty B + tz viz
-    const float aN = aChid * w.itz;
-    float aItz = aChid * w.N;
-    float aTx = aN * w.A, aTy = aN * w.Bv, aTz = aN * w.viz;
-    const float aA = aN * w.tx, aB = aN * w.ty;
-    float aViz = aN * w.tz;
-    aVix += aA;
-    aChi -= aA * wy;
-    ad.wy -= aA * w.chi;
-    aViy += aB;
-    aChi += aB * wx;
-    ad.wx += aB * w.chi;
-    // chi = Q itz, Q = (z - f) + (oz + zl)
-    const float aQ = aChi * w.itz;
-    aItz += aChi * w.Q;
-    ad.z += aQ;
-    float aF = -aQ;                                  // interpolated height
-    float aOz = aQ;
-    // itz = 1 / tz
-    aTz -= aItz * w.itz * w.itz;
-    // tau = R^T (-f_x, -f_y, 1)
-    ad.R[6] += aTx;
-    ad.R[0] -= aTx * w.t.y;
-    ad.R[3] -= aTx * w.t.z;
-    ad.R[7] += aTy;
-    ad.R[1] -= aTy * w.t.y;
-    ad.R[4] -= aTy * w.t.z;
-    ad.R[8] += aTz;
-    ad.R[2] -= aTz * w.t.y;
-    ad.R[5] -= aTz * w.t.z;
-    const float aGx = -(aTx * R[0] + aTy * R[1] + aTz * R[2]);   // interpolated f_x
-    const float aGy = -(aTx * R[3] + aTy * R[4] + aTz * R[5]);   // interpolated f_y
-    // bilinear: d/da = (1-b)(t10 - t00) + b (t11 - t01), d/db = hi - lo
-    const float4 &t00 = w.t00, &t10 = w.t10, &t01 = w.t01, &t11 = w.t11;
-    const float ob = 1.f - w.b, oa = 1.f - w.a;
-    const float dA_f = ob * (t10.x - t00.x) + w.b * (t11.x - t01.x);
-    const float dA_gx = ob * (t10.y - t00.y) + w.b * (t11.y - t01.y);
-    const float dA_gy = ob * (t10.z - t00.z) + w.b * (t11.z - t01.z);
-    const float dA_c = ob * (t10.w - t00.w) + w.b * (t11.w - t01.w);
-    const float dB_f = oa * (t01.x - t00.x) + w.a * (t11.x - t10.x);
-    const float dB_gx = oa * (t01.y - t00.y) + w.a * (t11.y - t10.y);
-    const float dB_gy = oa * (t01.z - t00.z) + w.a * (t11.z - t10.z);
-    const float dB_c = oa * (t01.w - t00.w) + w.a * (t11.w - t10.w);
-    const float aWa = aF * dA_f + aGx * dA_gx + aGy * dA_gy + aC * dA_c;
-    const float aWb = aF * dB_f + aGx * dB_gx + aGy * dB_gy + aC * dB_c;
-    float aOx = 0.f, aOy = 0.f;
-    if (!w.cx) {
-        ad.x += aWa * T.inv_cell;
-        aOx += aWa * T.inv_cell;
-    }
-    if (!w.cy) {
-        ad.y += aWb * T.inv_cell;
-        aOy += aWb * T.inv_cell;
-    }
-    // contact velocity v + w x rho, rho = (rx, ry, -(h+R))
-    ad.vx += aVix;
-    ad.wy -= aVix * V.hR;
-    ad.wz -= aVix * ry;
-    ad.vy += aViy;
-    ad.wz += aViy * rx;
-    ad.wx += aViy * V.hR;
-    ad.vz += aViz;
-    ad.wx += aViz * ry;
-    ad.wy -= aViz * rx;
-    // contact offset R rho
-    ad.R[0] += aOx * rx;
-    ad.R[1] += aOx * ry;
-    ad.R[2] -= aOx * V.hR;
-    ad.R[3] += aOy * rx;
-    ad.R[4] += aOy * ry;
-    ad.R[5] -= aOy * V.hR;
-    ad.R[6] += aOz * rx;
-    ad.R[7] += aOz * ry;
-    ad.R[8] -= aOz * V.hR;
 }
 
-struct StepOut {
-    float L;
-    bool stepped;     // false: the goal was reached before this step
+// dU_ESM / d(theta, phi): U = +/- M g Rbar (1 - (sin|phi| cos phibar + cos phi
+// sin phibar)) cos theta
+__device__ __forceinline__ void esm_grad(const Veh &V, float ph, float sth, float cth, float sph, float cph, float &th,
+                                         float &dph)
+{
+    const float sg = fabsf(ph) < V.tip ? V.MgRbar : -V.MgRbar;
+    const float sabs = ph < 0.f ? -sph : sph;
+    const float sv = fmaf(sabs, V.cpb, cph * V.spb);
+    th = -sg * (1.f - sv) * sth;
+    dph = -sg * cth * ((ph < 0.f ? -V.cpb : V.cpb) * cph - V.spb * sph);
+}
+
+struct BackParams {
+    Veh V;
+    Cost C;
+    Terrain T;
+    const float2 *ctrl;       // [H][K]
+    int K, H, n_sub;
+    float h;
+    int objective;
+    int k0, k1;               // this segment's control steps
+    int last, first;          // the rollout's last segment; its first
+    const float4 *rec;        // [K][(k1 - k0) n_sub][4]
+    const int *n_done, *emin;
+    const float4 *fin;
+    float *lam;               // [K][16] the adjoint between segments
+    float *grad;              // [H][K][2]
 };
 
-// One forward Euler step (the four-lane arithmetic of the plan kernel);
-// returns the running cost rate.
-__device__ __forceinline__ StepOut step_fwd(const GradParams &p, St &s, float dd, float ax, const Lane &ln)
+// The columns of Euler step e of candidate j into `out`.
+__device__ __forceinline__ void linearise(const BackParams &p, int j, int e, float *out)
 {
     const Veh &V = p.V;
     const Cost &Cc = p.C;
     const Terrain &T = p.T;
-    StepOut o;
-    o.L = 0.f;
-    o.stepped = false;
-    const float gdx = (s.x - Cc.gx_hi) + (s.xl - Cc.gx_lo);
-    const float gdy = (s.y - Cc.gy_hi) + (s.yl - Cc.gy_lo);
-    if (fmaf(gdx, gdx, gdy * gdy) <= Cc.goal_r2) return o;
-    o.stepped = true;
-    float sps, cps, sth, cth, sph, cph, sd, cd;
-    sincos_r(s.psi, sps, cps);
-    sincos_r(s.th, sth, cth);
-    sincos_r(s.ph, sph, cph);
-    sincos_r(s.d, sd, cd);
-    const float U = esm(V, s.ph, sph, cph, cth);
-    float R[9];
-    R[0] = cps * cth;
-    R[1] = fmaf(cps * sph, sth, -cph * sps);
-    R[2] = fmaf(cph * cps, sth, sph * sps);
-    R[3] = cth * sps;
-    R[4] = fmaf(sph * sps, sth, cph * cps);
-    R[5] = fmaf(cph * sps, sth, -cps * sph);
+    const float h = p.h;
+    const int n_rec = (p.k1 - p.k0) * p.n_sub;
+    const float4 *rec = p.rec + ((size_t)j * n_rec + (e - p.k0 * p.n_sub)) * 4;
+    const float4 s0 = rec[0], s1 = rec[1], s2 = rec[2], s3 = rec[3];
+    const float th = s1.w, ph = s2.x, d = s2.y, vx = s2.z, vy = s2.w, vz = s3.x, wx = s3.y, wy = s3.z, wz = s3.w;
+    const float2 u = __ldg(p.ctrl + (size_t)(e / p.n_sub) * p.K + j);
+    const bool inside = !(u.x < -V.ddmax || u.x > V.ddmax);       // as the clamp
+    const float dd = clamp_keep_nan(u.x, -V.ddmax, V.ddmax);
+    const float dn = fmaf(h, dd, d);
+    const bool d_clamped = dn < -V.dmax || dn > V.dmax;
+    Attitude A;
+    float sd, cd;
+    sincos_r(s1.z, A.sps, A.cps);
+    sincos_r(th, A.sth, A.cth);
+    sincos_r(ph, A.sph, A.cph);
+    sincos_r(d, sd, cd);
+    const float sth = A.sth, cth = A.cth, sph = A.sph, cph = A.cph;
+    float *R = A.R;
+    R[0] = A.cps * cth;
+    R[1] = fmaf(A.cps * sph, sth, -cph * A.sps);
+    R[2] = fmaf(cph * A.cps, sth, sph * A.sps);
+    R[3] = cth * A.sps;
+    R[4] = fmaf(sph * A.sps, sth, cph * A.cps);
+    R[5] = fmaf(cph * A.sps, sth, -A.cps * sph);
     R[6] = -sth;
     R[7] = cth * sph;
     R[8] = cph * cth;
-    const Cell cx = cell_of<false>(s.x, s.xl, T.inv_cell, T.nx), cy = cell_of<false>(s.y, s.yl, T.inv_cell, T.ny);
+    const Cell cx = cell_of<false>(s0.x, s0.y, T.inv_cell, T.nx), cy = cell_of<false>(s0.z, s0.w, T.inv_cell, T.ny);
     const unsigned base = texel_base(cx, cy, T.nx);
-    const float gBx = -V.g * R[6], gBy = -V.g * R[7], gBz = -V.g * R[8];
-    WF w;
-    wheel_fwd(V, T, R, cx, cy, base, s.z, s.zl, s.vx, s.vy, s.vz, s.wx, s.wy, s.wz, ln.rx, ln.ry, ln.k,
-              ln.b, ln.Fs, ln.front ? s.d : 0.f, w);
-    const float fy = ln.front ? w.Fy * cd : w.Fy;
-    const float FyB = qsum(fy, ln.mask);
-    const float FzB = qsum(w.Fz, ln.mask);
-    const float Mx = fmaf(V.hR, FyB, qsum(ln.ry * w.Fz, ln.mask));
-    float My = qsum(-ln.rx * w.Fz, ln.mask);
-    const float Mz = qsum(ln.rx * fy, ln.mask);
-    const float csum = T.has_cm ? qsum(w.t.w, ln.mask) : 0.f;
-    const float Fx = V.halfM * fmaf(-s.wz, s.vy, fmaf(s.wy, s.vz, ax - gBx));
-    My = fmaf(-V.hR, 2.f * Fx, My);
+
+    // gradients of the five force sums S = sum F_y (turned by delta in front),
+    // sum F_z, sum r_y F_z, sum -r_x F_z, sum r_x F_y
+    float S[5][12], Sd0 = 0.f, Sd4 = 0.f, cg[6];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) S[0][c] = S[1][c] = S[2][c] = S[3][c] = S[4][c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) cg[c] = 0.f;
+#pragma unroll 1
+    for (int i = 0; i < 4; ++i) {
+        const bool front = i < 2;
+        const float rx = front ? V.Lf : -V.Lr, ry = (i & 1) ? -V.he : V.he;
+        WheelGrad w;
+        wheel_lin(V, T, A, cx, cy, base, s1.x, s1.y, vx, vy, vz, wx, wy, wz, rx, ry, front ? V.kf : V.kr,
+                  front ? V.bf : V.br, front ? V.Fsf : V.Fsr, front ? d : 0.f, w);
+        const float turn = front ? cd : 1.f;
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            float fy = w.ratio * w.g[c];
+            if (c == 6) fy += w.a[0];
+            if (c == 7) fy += w.a[1];
+            if (c >= 9) fy += w.a[c - 7];
+            fy *= turn;
+            S[0][c] += fy;
+            S[1][c] += w.g[c];
+            S[2][c] = fmaf(ry, w.g[c], S[2][c]);
+            S[3][c] = fmaf(-rx, w.g[c], S[3][c]);
+            S[4][c] = fmaf(rx, fy, S[4][c]);
+        }
+        if (front) {
+            const float fd = fmaf(w.ad, cd, -sd * w.Fy);
+            Sd0 += fd;
+            Sd4 = fmaf(rx, fd, Sd4);
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) cg[c] += w.c[c];
+    }
+    // the force rows of the step's matrix (times the Euler step): y and z
+    // velocity, then the rates by Euler's equations
+    const float kv = h * V.invM, kx = h * V.invJxx, ky = h * V.invJyy, kz = h * V.invJzz;
+    const float fx = -2.f * V.hR * ky * V.halfM;            // the rear constraint force in My
+    float D[5][12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        D[0][c] = kv * S[0][c];
+        D[1][c] = kv * S[1][c];
+        D[2][c] = kx * fmaf(V.hR, S[0][c], S[2][c]);
+        D[3][c] = ky * S[3][c];
+        D[4][c] = kz * S[4][c];
+    }
+    const float hg = h * V.g;
+    D[0][4] = fmaf(hg, sth * sph, D[0][4]);                 // gravity in B
+    D[0][5] = fmaf(-hg, cth * cph, D[0][5]);
+    D[1][4] = fmaf(hg, cph * sth, D[1][4]);
+    D[1][5] = fmaf(hg, sph * cth, D[1][5]);
+    D[3][4] = fmaf(-fx * V.g, cth, D[3][4]);
+    D[0][6] = fmaf(-h, wz, D[0][6]);                        // the velocities' cross terms
+    D[0][8] = fmaf(h, wx, D[0][8]);
+    D[0][9] = fmaf(h, vz, D[0][9]);
+    D[0][11] = fmaf(-h, vx, D[0][11]);
+    D[1][6] = fmaf(h, wy, D[1][6]);
+    D[1][7] = fmaf(-h, wx, D[1][7]);
+    D[1][9] = fmaf(-h, vy, D[1][9]);
+    D[1][10] = fmaf(h, vx, D[1][10]);
+    D[2][10] = fmaf(kx * V.dJyz, wz, D[2][10]);
+    D[2][11] = fmaf(kx * V.dJyz, wy, D[2][11]);
+    D[3][7] = fmaf(-fx, wz, D[3][7]);
+    D[3][8] = fmaf(fx, wy, D[3][8]);
+    D[3][9] = fmaf(-ky * V.dJxz, wz, D[3][9]);
+    D[3][10] = fmaf(fx, vz, D[3][10]);
+    D[3][11] = fmaf(-ky * V.dJxz, wx, fmaf(-fx, vy, D[3][11]));
+    D[4][9] = fmaf(kz * V.dJxy, wy, D[4][9]);
+    D[4][10] = fmaf(kz * V.dJxy, wx, D[4][10]);
+
+    // the constants: the running cost's gradient, or the margin's at its state
+    const float sv = fmaf(ph < 0.f ? -sph : sph, V.cpb, cph * V.spb);
+    const float uu = V.MgRbar * (1.f - sv) * cth;
+    const float U = fabsf(ph) < V.tip ? uu : -uu;
     const float soft = fmaxf(fmaf(-U, Cc.inv_eps, 1.f), 0.f);
-    o.L = fmaf(Cc.sigma * soft, soft, fmaf(Cc.wc * dd, dd, Cc.wt)) + csum;
+    float eth, eph;
+    esm_grad(V, ph, sth, cth, sph, cph, eth, eph);
+    const bool cost = p.objective == kGradCost;
+    const float aU = cost ? (soft > 0.f ? -h * 2.f * Cc.sigma * soft * Cc.inv_eps : 0.f)
+                          : (e == p.emin[j] ? 1.f : 0.f);
+    const float hc = cost ? h : 0.f;
+    float cst[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) cst[c] = hc * cg[c];
+    if (aU != 0.f) {
+        cst[4] = fmaf(aU, eth, cst[4]);
+        cst[5] = fmaf(aU, eph, cst[5]);
+    }
+
+    // the kinematic rows, and every column into shared memory
     const float ic = rcp(cth);
-    const float wsc = fmaf(sph, s.wy, cph * s.wz);
-    const float dx = fmaf(R[2], s.vz, fmaf(R[1], s.vy, R[0] * s.vx));
-    const float dy = fmaf(R[5], s.vz, fmaf(R[4], s.vy, R[3] * s.vx));
-    const float dz = fmaf(R[8], s.vz, fmaf(R[7], s.vy, R[6] * s.vx));
-    const float dpsi = wsc * ic;
-    const float dth = fmaf(cph, s.wy, -sph * s.wz);
-    const float dph = fmaf(wsc, sth * ic, s.wx);
-    const float dvy = fmaf(-s.wz, s.vx, fmaf(s.wx, s.vz, fmaf(FyB, V.invM, gBy)));
-    const float dvz = fmaf(s.wy, s.vx, fmaf(-s.wx, s.vy, fmaf(FzB, V.invM, gBz)));
-    const float dwx = fmaf(V.dJyz * s.wy, s.wz, Mx) * V.invJxx;
-    const float dwy = fmaf(-V.dJxz * s.wx, s.wz, My) * V.invJyy;
-    const float dwz = fmaf(V.dJxy * s.wx, s.wy, Mz) * V.invJzz;
-    const float h = p.h;
-    acc2(s.x, s.xl, h * dx);
-    acc2(s.y, s.yl, h * dy);
-    acc2(s.z, s.zl, h * dz);
-    acc2(s.psi, s.psil, h * dpsi);
-    s.th = fmaf(h, dth, s.th);
-    s.ph = fmaf(h, dph, s.ph);
-    acc2(s.vx, s.vxl, h * ax);
-    acc2(s.vy, s.vyl, h * dvy);
-    acc2(s.vz, s.vzl, h * dvz);
-    s.wx = fmaf(h, dwx, s.wx);
-    s.wy = fmaf(h, dwy, s.wy);
-    s.wz = fmaf(h, dwz, s.wz);
-    s.d = clampf(fmaf(h, dd, s.d), -V.dmax, V.dmax);
-    return o;
+    const float wsc = fmaf(sph, wy, cph * wz), wdf = fmaf(cph, wy, -sph * wz);
+    const float bth = fmaf(sph, vy, cph * vz);              // along dR / d(theta)
+    const float xth = fmaf(cth, bth, -sth * vx), zth = -fmaf(sth, bth, cth * vx);
+    float4 *o = (float4 *)out;
+    const auto column = [&](int c, float x, float y, float z, float ps, float t, float f, float k) {
+        o[4 * c] = make_float4(x, y, z, ps);
+        o[4 * c + 1] = make_float4(t, f, 0.f, D[0][c]);
+        o[4 * c + 2] = make_float4(D[1][c], D[2][c], D[3][c], D[4][c]);
+        o[4 * c + 3] = make_float4(0.f, k, 0.f, 1.f);
+    };
+    column(X, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, cst[0]);
+    column(Y, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, cst[1]);
+    column(Z, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, cst[2]);
+    column(PSI, -h * fmaf(R[5], vz, fmaf(R[4], vy, R[3] * vx)), h * fmaf(R[2], vz, fmaf(R[1], vy, R[0] * vx)), 0.f, 0.f,
+           0.f, 0.f, cst[3]);
+    column(TH, h * A.cps * xth, h * A.sps * xth, h * zth, h * wsc * sth * ic * ic, 0.f,
+           h * wsc * fmaf(sth * ic, sth * ic, cth * ic), cst[4]);
+    column(PH, h * fmaf(R[2], vy, -R[1] * vz), h * fmaf(R[5], vy, -R[4] * vz), h * fmaf(R[8], vy, -R[7] * vz),
+           h * ic * wdf, -h * wsc, h * sth * ic * wdf, cst[5]);
+    column(VX, h * R[0], h * R[3], h * R[6], 0.f, 0.f, 0.f, 0.f);
+    column(VY, h * R[1], h * R[4], h * R[7], 0.f, 0.f, 0.f, 0.f);
+    column(VZ, h * R[2], h * R[5], h * R[8], 0.f, 0.f, 0.f, 0.f);
+    column(WX, 0.f, 0.f, 0.f, 0.f, 0.f, h, 0.f);
+    column(WY, 0.f, 0.f, 0.f, h * sph * ic, h * cph, h * sph * sth * ic, 0.f);
+    column(WZ, 0.f, 0.f, 0.f, h * cph * ic, -h * sph, h * cph * sth * ic, 0.f);
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    o[4 * DE] = zero;
+    o[4 * DE + 1] = make_float4(0.f, 0.f, 0.f, kv * Sd0);
+    o[4 * DE + 2] = make_float4(0.f, kx * V.hR * Sd0, 0.f, kz * Sd4);
+    o[4 * DE + 3] = make_float4(0.f, 0.f, 0.f, d_clamped ? 0.f : 1.f);
+    o[4 * kGdd] = zero;
+    o[4 * kGdd + 1] = zero;
+    o[4 * kGdd + 2] = zero;
+    o[4 * kGdd + 3] = make_float4(d_clamped ? 0.f : h, hc * 2.f * Cc.wc * dd, inside ? 1.f : 0.f, 1.f);
+    o[4 * kGax] = zero;
+    o[4 * kGax + 1] = make_float4(0.f, 0.f, h, 0.f);
+    o[4 * kGax + 2] = make_float4(0.f, 0.f, fx, 0.f);
+    o[4 * kGax + 3] = make_float4(0.f, 0.f, 0.f, 1.f);
 }
 
-// One Euler step backwards from the state s at its start: lam (13: x, y, z,
-// psi, theta, phi, vx, vy, vz, wx, wy, wz, delta) is the adjoint of the state
-// after the step on entry and of the state before it on exit; g_dd and g_ax
-// receive the step's contributions to dJ/d(steering rate) and dJ/d(accel).
-__device__ void step_adj(const GradParams &p, const St &s, float dd, float ax, float lam[13], float &g_dd,
-                         float &g_ax, const Lane &ln)
+// The recursion over n steps from the last to step e of `mats`, this lane's
+// column of each: returns the adjoint (and the open gradients) before them.
+// SPAN lanes run one candidate; candidates with fewer steps than the warp's
+// longest sit out the rest.  The adjoint goes round through 16 floats of
+// shared memory, in turn the two of `turn`: one store and four broadcast loads
+// a step, where 13 shuffles took twice the time.  GUARD leaves out the
+// matrix's zeros, which a NaN would pass through.
+template <int SPAN, bool GUARD>
+__device__ __forceinline__ float recursion(const BackParams &p, int j, const float *mats, float *turn, int e, int n,
+                                           int lane, float lam)
 {
-    // the running cost enters the cost's adjoint only
-    const float cw = p.objective == kGradCost ? 1.f : 0.f;
-    const Veh &V = p.V;
-    const Cost &Cc = p.C;
-    const Terrain &T = p.T;
-    const float h = p.h;
-    float sps, cps, sth, cth, sph, cph, sd, cd;
-    sincos_r(s.psi, sps, cps);
-    sincos_r(s.th, sth, cth);
-    sincos_r(s.ph, sph, cph);
-    sincos_r(s.d, sd, cd);
-    const float U = esm(V, s.ph, sph, cph, cth);
-    float R[9];
-    R[0] = cps * cth;
-    R[1] = fmaf(cps * sph, sth, -cph * sps);
-    R[2] = fmaf(cph * cps, sth, sph * sps);
-    R[3] = cth * sps;
-    R[4] = fmaf(sph * sps, sth, cph * cps);
-    R[5] = fmaf(cph * sps, sth, -cps * sph);
-    R[6] = -sth;
-    R[7] = cth * sph;
-    R[8] = cph * cth;
-    const Cell cx = cell_of<false>(s.x, s.xl, T.inv_cell, T.nx), cy = cell_of<false>(s.y, s.yl, T.inv_cell, T.ny);
-    const unsigned base = texel_base(cx, cy, T.nx);
-    const float vx = s.vx, vy = s.vy, vz = s.vz, wx = s.wx, wy = s.wy, wz = s.wz;
-    WF w;
-    wheel_fwd(V, T, R, cx, cy, base, s.z, s.zl, vx, vy, vz, wx, wy, wz, ln.rx, ln.ry, ln.k, ln.b, ln.Fs,
-              ln.front ? s.d : 0.f, w);
-    const float soft = fmaxf(fmaf(-U, Cc.inv_eps, 1.f), 0.f);
-    const float ic = rcp(cth);
-    const float wsc = fmaf(sph, wy, cph * wz);
-    const float dd_next = fmaf(h, dd, s.d);
-    const bool d_clamped = dd_next < -V.dmax || dd_next > V.dmax;
-
-    Adj ad;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) ad.R[c] = 0.f;
-    // Euler update: state' = state + h * rate
-    ad.x = lam[0];
-    ad.y = lam[1];
-    ad.z = lam[2];
-    float a_psi = lam[3], a_th = lam[4], a_ph = lam[5];
-    ad.vx = lam[6];
-    ad.vy = lam[7];
-    ad.vz = lam[8];
-    ad.wx = lam[9];
-    ad.wy = lam[10];
-    ad.wz = lam[11];
-    float a_d = d_clamped ? 0.f : lam[12];
-    const float a_dx = h * lam[0], a_dy = h * lam[1], a_dz = h * lam[2];
-    const float a_dpsi = h * lam[3], a_dth = h * lam[4], a_dph = h * lam[5];
-    g_ax += h * lam[6];
-    const float a_dvy = h * lam[7], a_dvz = h * lam[8];
-    const float a_dwx = h * lam[9], a_dwy = h * lam[10], a_dwz = h * lam[11];
-    if (!d_clamped) g_dd += h * lam[12];
-    // running cost: J += h L, L = wt + wc dd^2 + sigma soft^2 + sum of costmap
-    g_dd += cw * (h * 2.f * Cc.wc * dd);
-    float a_U = 0.f;
-    if (soft > 0.f) a_U = cw * (-h * 2.f * Cc.sigma * soft * Cc.inv_eps);
-    const float a_csum = cw * h;
-    // positions: d(x,y,z) = R v
-    float a_sph = 0.f, a_cph = 0.f, a_sth = 0.f, a_cth = 0.f, a_sps = 0.f, a_cps = 0.f;
-    ad.R[0] += a_dx * vx; ad.R[1] += a_dx * vy; ad.R[2] += a_dx * vz;
-    ad.R[3] += a_dy * vx; ad.R[4] += a_dy * vy; ad.R[5] += a_dy * vz;
-    ad.R[6] += a_dz * vx; ad.R[7] += a_dz * vy; ad.R[8] += a_dz * vz;
-    ad.vx += a_dx * R[0] + a_dy * R[3] + a_dz * R[6];
-    ad.vy += a_dx * R[1] + a_dy * R[4] + a_dz * R[7];
-    ad.vz += a_dx * R[2] + a_dy * R[5] + a_dz * R[8];
-    // Euler-angle rates
-    const float a_wsc = a_dpsi * ic + a_dph * sth * ic;
-    const float a_ic = a_dpsi * wsc + a_dph * wsc * sth;
-    a_sth += a_dph * wsc * ic;
-    ad.wx += a_dph;
-    a_cph += a_dth * wy;
-    ad.wy += a_dth * cph;
-    a_sph -= a_dth * wz;
-    ad.wz -= a_dth * sph;
-    a_sph += a_wsc * wy;
-    ad.wy += a_wsc * sph;
-    a_cph += a_wsc * wz;
-    ad.wz += a_wsc * cph;
-    a_cth -= a_ic * ic * ic;
-    // velocity rates
-    const float a_FyB0 = a_dvy * V.invM;
-    const float a_gBy = a_dvy;
-    ad.wx += a_dvy * vz;
-    ad.vz += a_dvy * wx;
-    ad.wz -= a_dvy * vx;
-    ad.vx -= a_dvy * wz;
-    const float a_FzB = a_dvz * V.invM;
-    const float a_gBz = a_dvz;
-    ad.wx -= a_dvz * vy;
-    ad.vy -= a_dvz * wx;
-    ad.wy += a_dvz * vx;
-    ad.vx += a_dvz * wy;
-    // angular rates (Euler's equations)
-    const float a_Mx = a_dwx * V.invJxx, a_My = a_dwy * V.invJyy, a_Mz = a_dwz * V.invJzz;
-    ad.wy += a_Mx * V.dJyz * wz;
-    ad.wz += a_Mx * V.dJyz * wy;
-    ad.wx -= a_My * V.dJxz * wz;
-    ad.wz -= a_My * V.dJxz * wx;
-    ad.wx += a_Mz * V.dJxy * wy;
-    ad.wy += a_Mz * V.dJxy * wx;
-    // rear longitudinal constraint force, which enters My only
-    const float a_Fx = -2.f * V.hR * a_My;
-    g_ax += a_Fx * V.halfM;
-    float a_gBx = -a_Fx * V.halfM;
-    ad.wy += a_Fx * V.halfM * vz;
-    ad.vz += a_Fx * V.halfM * wy;
-    ad.wz -= a_Fx * V.halfM * vy;
-    ad.vy -= a_Fx * V.halfM * wz;
-    // sums: FyB = sum fy, Mx = hR FyB + sum ry Fz, My = sum -rx Fz (+ the
-    // constraint force), Mz = sum rx fy, with fy = Fy cos(delta) in front
-    const float a_FyB = a_FyB0 + V.hR * a_Mx;
-    const float a_fy = a_FyB + ln.rx * a_Mz;
-    const float aFy = ln.front ? a_fy * cd : a_fy;
-    const float aFz = a_FzB + ln.ry * a_Mx - ln.rx * a_My;
-    // gravity in B
-    ad.R[6] -= V.g * a_gBx;
-    ad.R[7] -= V.g * a_gBy;
-    ad.R[8] -= V.g * a_gBz;
-    // this lane's wheel into its own accumulator, then the quad's sum
-    Adj aw;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) aw.R[c] = 0.f;
-    aw.x = aw.y = aw.z = aw.vx = aw.vy = aw.vz = aw.wx = aw.wy = aw.wz = aw.d = 0.f;
-    float a_dw = ln.front ? -sd * a_fy * w.Fy : 0.f;                // cos(delta) of the front forces
-    wheel_adj(V, T, R, wx, wy, ln.rx, ln.ry, ln.k, ln.b, ln.front ? 1.f : 0.f, w, aFz, aFy, a_csum, aw, a_dw);
-#pragma unroll
-    for (int c = 0; c < 9; ++c) ad.R[c] += qsum(aw.R[c], ln.mask);
-    ad.x += qsum(aw.x, ln.mask);
-    ad.y += qsum(aw.y, ln.mask);
-    ad.z += qsum(aw.z, ln.mask);
-    ad.vx += qsum(aw.vx, ln.mask);
-    ad.vy += qsum(aw.vy, ln.mask);
-    ad.vz += qsum(aw.vz, ln.mask);
-    ad.wx += qsum(aw.wx, ln.mask);
-    ad.wy += qsum(aw.wy, ln.mask);
-    ad.wz += qsum(aw.wz, ln.mask);
-    a_d += qsum(a_dw, ln.mask);
-    // ESM: U = +/- M g Rbar (1 - (sin|phi| cos phibar + cos phi sin phibar)) cos theta
-    {
-        const float sg = fabsf(s.ph) < V.tip ? 1.f : -1.f;
-        const float sabs = s.ph < 0.f ? -sph : sph;
-        const float sv = fmaf(sabs, V.cpb, cph * V.spb);
-        const float a_u = sg * a_U;
-        const float a_s = -V.MgRbar * cth * a_u;
-        a_cth += V.MgRbar * (1.f - sv) * a_u;
-        a_sph += (s.ph < 0.f ? -1.f : 1.f) * a_s * V.cpb;
-        a_cph += a_s * V.spb;
-    }
-    // rotation matrix
-    const float *aR = ad.R;
-    a_cps += aR[0] * cth + aR[1] * sph * sth + aR[2] * cph * sth + aR[4] * cph - aR[5] * sph;
-    a_cth += aR[0] * cps + aR[3] * sps + aR[7] * sph + aR[8] * cph;
-    a_sph += aR[1] * cps * sth + aR[2] * sps + aR[4] * sps * sth - aR[5] * cps + aR[7] * cth;
-    a_sth += aR[1] * cps * sph + aR[2] * cph * cps + aR[4] * sph * sps + aR[5] * cph * sps - aR[6];
-    a_cph += -aR[1] * sps + aR[2] * cps * sth + aR[4] * cps + aR[5] * sps * sth + aR[8] * cth;
-    a_sps += -aR[1] * cph + aR[2] * sph + aR[3] * cth + aR[4] * sph * sth + aR[5] * cph * sth;
-    // angles
-    a_psi += a_sps * cps - a_cps * sps;
-    a_th += a_sth * cth - a_cth * sth;
-    a_ph += a_sph * cph - a_cph * sph;
-    lam[0] = ad.x;
-    lam[1] = ad.y;
-    lam[2] = ad.z;
-    lam[3] = a_psi;
-    lam[4] = a_th;
-    lam[5] = a_ph;
-    lam[6] = ad.vx;
-    lam[7] = ad.vy;
-    lam[8] = ad.vz;
-    lam[9] = ad.wx;
-    lam[10] = ad.wy;
-    lam[11] = ad.wz;
-    lam[12] = a_d;
-}
-
-// U_ESM of a state (Sec. IV-B), as the plan kernel evaluates it
-__device__ __forceinline__ float state_esm(const Veh &V, const St &s)
-{
-    float sth, cth, sph, cph;
-    sincos_r(s.th, sth, cth);
-    sincos_r(s.ph, sph, cph);
-    return esm(V, s.ph, sph, cph, cth);
-}
-
-// lam += dU_ESM/d(state) at the state s: U = +/- M g Rbar (1 - (sin|phi|
-// cos phibar + cos phi sin phibar)) cos theta depends on theta and phi only
-__device__ __forceinline__ void esm_adj(const Veh &V, const St &s, float lam[13])
-{
-    float sth, cth, sph, cph;
-    sincos_r(s.th, sth, cth);
-    sincos_r(s.ph, sph, cph);
-    const float sg = fabsf(s.ph) < V.tip ? 1.f : -1.f;
-    const float sabs = s.ph < 0.f ? -sph : sph;
-    const float sv = fmaf(sabs, V.cpb, cph * V.spb);
-    const float a_s = -V.MgRbar * cth * sg;
-    const float a_cth = V.MgRbar * (1.f - sv) * sg;
-    const float a_sph = (s.ph < 0.f ? -1.f : 1.f) * a_s * V.cpb;
-    const float a_cph = a_s * V.spb;
-    lam[4] -= a_cth * sth;
-    lam[5] += a_sph * cph - a_cph * sph;
-}
-
-// The forward pass stores the checkpoints and the last segment's Euler-step
-// start states.  Then round i walks segment n_seg - 1 - i backwards and
-// recomputes the segment before it.
-//   SPLIT = false: one quad per candidate walks, then recomputes into the
-//   buffer it has just read (one buffer).
-//   SPLIT = true (a grid that leaves most of the GPU idle): each CTA holds
-//   its kGradCands candidates twice.  Its first half of threads walks, its
-//   second half recomputes, both having run the forward pass (the same
-//   bits), so the recomputation runs beside the walk instead of before it,
-//   into the other of two buffers.  A CTA barrier ends each round; every
-//   thread, a candidate-less one included, passes the same number of
-//   barriers (n_seg, uniform over the grid).
-template <bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? 2 * kGradHalf : kGradHalf, 1) grad_kernel(const __grid_constant__ GradParams p)
-{
-    const bool walker = !SPLIT || threadIdx.x < kGradHalf;
-    const bool recomp = !SPLIT || !walker;
-    const int tid = blockIdx.x * kGradHalf + (threadIdx.x & (kGradHalf - 1));   // lane slot, either half
-    const int j = tid / kGradLanes;
-    const bool active = j < p.K;                // whole quads, in both halves alike
-    const Lane ln = lane_of(p.V, tid & (kGradLanes - 1), 0xfu << (threadIdx.x & 28));
-    const Terrain &T = p.T;
-    const Cost &Cc = p.C;
-    const size_t K = (size_t)p.K;
-    const size_t KL = K * kGradLanes;           // every lane keeps its own copy of the states
-    const int n_seg = (p.H + p.ckpt - 1) / p.ckpt;
-    const int k_last = (n_seg - 1) * p.ckpt;    // first control step of the last segment
-    const size_t seg_stride = (size_t)p.ckpt * p.n_sub * kStFloats * KL;
-    float *ck = p.ckpt_buf + tid;               // [n_seg][20][K lanes]
-    float *seg = p.seg_buf + tid;               // [1 or 2][ckpt * n_sub][20][K lanes]
-    const bool want_margin = p.objective == kGradMargin;
-    St s;
-    float J = 0.f;
-    float Umin = CUDART_INF_F;                   // the margin: min U_ESM over the states
-    int emin = 0;                                // index of the state holding it (first on ties)
-    int done_step = p.H * p.n_sub;               // Euler step index where the goal stopped the rollout
-    float lam[13];
-#pragma unroll
-    for (int c = 0; c < 13; ++c) lam[c] = 0.f;
-    if (active) {
-        {
-            float q[13];
-            if (p.x0_soa) {
-#pragma unroll
-                for (int c = 0; c < 13; ++c) q[c] = p.x0_soa[c * K + j];
-            } else {
-#pragma unroll
-                for (int c = 0; c < 13; ++c) q[c] = p.x0[c];
-            }
-            two_sum(q[0], -T.x0_hi, s.x, s.xl);
-            s.xl -= T.x0_lo;
-            two_sum(q[1], -T.y0_hi, s.y, s.yl);
-            s.yl -= T.y0_lo;
-            s.z = q[2]; s.psi = q[3]; s.th = q[4]; s.ph = q[5];
-            s.vx = q[6]; s.vy = q[7]; s.vz = q[8];
-            s.wx = q[9]; s.wy = q[10]; s.wz = q[11]; s.d = q[12];
-            s.zl = s.psil = s.vxl = s.vyl = s.vzl = 0.f;
+    const int col = lane < kCols ? lane : kCols - 1;
+    const int n_max = SPAN == 32 ? n : max(n, __shfl_xor_sync(kFull, n, 16));
+    int k = (e + n - 1) / p.n_sub, sub = (e + n - 1) - k * p.n_sub;
+    const float4 *m = (const float4 *)mats + (size_t)max(n - 1, 0) * (kStepFloats / 4) + 4 * col;
+    float4 a = m[0], b = m[1], c = m[2], d = m[3];
+    for (int s = 0; s < n_max; ++s) {
+        float *l = turn + (s & 1) * 16;
+        if (SPAN == 16 || lane < 16) l[lane] = lam;
+        const float4 a0 = a, b0 = b, c0 = c, d0 = d;
+        if (s + 1 < n) {                                    // the next step's column, ahead
+            m -= kStepFloats / 4;
+            a = m[0]; b = m[1]; c = m[2]; d = m[3];
         }
-        // forward: cost (or margin), checkpoints and the last segment's states
-        bool done = false;
-        for (int k = 0; k < p.H; ++k) {
-            if (recomp && k % p.ckpt == 0) st_store(ck + (size_t)(k / p.ckpt) * kStFloats * KL, KL, s);
-            const float2 u = __ldg(p.ctrl + (size_t)k * K + j);
-            const float dd = clampf(u.x, -p.V.ddmax, p.V.ddmax);
-            for (int q = 0; q < p.n_sub && !done; ++q) {
-                if (recomp && k >= k_last)
-                    st_store(seg + (size_t)((k - k_last) * p.n_sub + q) * kStFloats * KL, KL, s);
-                if (want_margin) {
-                    const float U = state_esm(p.V, s);
-                    if (U < Umin) {
-                        Umin = U;
-                        emin = k * p.n_sub + q;
-                    }
-                }
-                const StepOut o = step_fwd(p, s, dd, u.y, ln);
-                if (!o.stepped) {
-                    done = true;
-                    done_step = k * p.n_sub + q;
-                    break;
-                }
-                J = fmaf(p.h, o.L, J);
-            }
-        }
-        // terminal cost and its gradient, or the final state's share of the margin
-        if (walker) {
-            if (want_margin) {
-                const int e_final = done ? done_step : p.H * p.n_sub;
-                const float U = state_esm(p.V, s);
-                if (U < Umin) {
-                    Umin = U;
-                    emin = e_final;
-                }
-                if (emin == e_final) esm_adj(p.V, s, lam);
-                if (ln.q == 0) p.cost[j] = Umin;
-            } else {
-                const float gdx = (s.x - Cc.gx_hi) + (s.xl - Cc.gx_lo);
-                const float gdy = (s.y - Cc.gy_hi) + (s.yl - Cc.gy_lo);
-                const float dist = sqrtf(fmaf(gdx, gdx, gdy * gdy));
-                J = fmaf(Cc.wg, dist, J);
-                if (ln.q == 0) p.cost[j] = J;
-                if (dist > 0.f) {
-                    lam[0] = Cc.wg * gdx / dist;
-                    lam[1] = Cc.wg * gdy / dist;
-                }
+        __syncwarp();
+        const float4 la = ((const float4 *)l)[0], lb = ((const float4 *)l)[1], lc = ((const float4 *)l)[2];
+        const float ld = l[DE];
+        const auto add = [](float w, float v, float q) { return GUARD && w == 0.f ? q : fmaf(w, v, q); };
+        float q0 = add(a0.x, la.x, d0.y), q1 = add(a0.y, la.y, 0.f), q2 = add(a0.z, la.z, 0.f), q3 = add(a0.w, la.w, 0.f);
+        q0 = add(b0.x, lb.x, q0);
+        q1 = add(b0.y, lb.y, q1);
+        q2 = add(b0.z, lb.z, q2);
+        q3 = add(b0.w, lb.w, q3);
+        q0 = add(c0.x, lc.x, q0);
+        q1 = add(c0.y, lc.y, q1);
+        q2 = add(c0.z, lc.z, q2);
+        q3 = add(c0.w, lc.w, q3);
+        q0 = add(d0.x, ld, q0);
+        const float q = (q0 + q1) + (q2 + q3);
+        if (SPAN == 32 || s < n) {
+            lam = GUARD && d0.w == 0.f ? q : fmaf(d0.w, lam, q);
+            if (sub-- == 0) {                               // the control step is complete
+                if (lane == kGdd || lane == kGax)
+                    p.grad[((size_t)k * p.K + j) * 2 + (lane - kGdd)] = lane == kGdd && d0.z == 0.f ? 0.f : lam;
+                if (lane >= kGdd) lam = 0.f;
+                --k;
+                sub = p.n_sub - 1;
             }
         }
     }
-    if (SPLIT) __syncthreads();                 // the last segment's states are stored
-    // reverse: round i walks segment n_seg - 1 - i and recomputes the one before it
-    for (int i = 0; i < n_seg; ++i) {
-        const int sw = n_seg - 1 - i;
-        if (active && walker) {
-            const int k0 = sw * p.ckpt, k1 = min(p.H, k0 + p.ckpt);
-            const float *buf = SPLIT ? seg + (size_t)(i & 1) * seg_stride : seg;
-            for (int k = k1 - 1; k >= k0; --k) {
-                const float2 u = __ldg(p.ctrl + (size_t)k * K + j);
-                const bool inside = !(u.x < -p.V.ddmax || u.x > p.V.ddmax);   // as the clamp
-                const float dd = clampf(u.x, -p.V.ddmax, p.V.ddmax);
-                float g_dd = 0.f, g_ax = 0.f;
-                for (int q = p.n_sub - 1; q >= 0; --q) {
-                    const int e = k * p.n_sub + q;
-                    if (e >= done_step) continue;
-                    St r2;
-                    st_load(buf + (size_t)(e - k0 * p.n_sub) * kStFloats * KL, KL, r2);
-                    step_adj(p, r2, dd, u.y, lam, g_dd, g_ax, ln);
-                    // lam is now the adjoint of the step's start state
-                    if (want_margin && e == emin) esm_adj(p.V, r2, lam);
-                }
-                // the steering rate is clamped to +/- its limit before use
-                if (ln.q == 0) {
-                    p.grad[((size_t)k * K + j) * 2] = inside ? g_dd : 0.f;
-                    p.grad[((size_t)k * K + j) * 2 + 1] = g_ax;
-                }
-            }
-        }
-        if (active && recomp && sw > 0) {
-            // recompute segment sw - 1's Euler-step start states
-            const int sr = sw - 1;
-            const int k0 = sr * p.ckpt, k1 = k0 + p.ckpt;                 // never the last segment
-            float *buf = SPLIT ? seg + (size_t)((i + 1) & 1) * seg_stride : seg;
-            St r;
-            st_load(ck + (size_t)sr * kStFloats * KL, KL, r);
-            int n_steps = 0;
-            for (int k = k0; k < k1; ++k) {
-                const float2 u = __ldg(p.ctrl + (size_t)k * K + j);
-                const float dd = clampf(u.x, -p.V.ddmax, p.V.ddmax);
-                for (int q = 0; q < p.n_sub; ++q) {
-                    const int e = k * p.n_sub + q;
-                    if (e >= done_step) break;
-                    st_store(buf + (size_t)n_steps * kStFloats * KL, KL, r);
-                    ++n_steps;
-                    step_fwd(p, r, dd, u.y, ln);
-                }
-            }
-        }
-        if (SPLIT && i + 1 < n_seg) __syncthreads();   // segment sw - 1 is stored; segment sw is read
+    __syncwarp();
+    return lam;
+}
+
+// a chunk's recursion; a diverged rollout's infinities and NaN pass only
+// through the entries the steps' matrices have
+template <int SPAN>
+__device__ __forceinline__ float run_chunk(const BackParams &p, int j, const float *mats, float *turn, int e, int n,
+                                           int lane, float lam)
+{
+    const float out = recursion<SPAN, false>(p, j, mats, turn, e, n, lane, lam);
+    return __any_sync(kFull, !isfinite(out)) ? recursion<SPAN, true>(p, j, mats, turn, e, n, lane, lam) : out;
+}
+
+// What the recursion of candidate j starts from; lane is the component.
+__device__ __forceinline__ float first_lam(const BackParams &p, int j, int n_done, int lane)
+{
+    float lam = 0.f;
+    if (!p.last) return lane < kRows ? p.lam[(size_t)j * 16 + lane] : 0.f;
+    const float4 f = p.fin[j];
+    if (p.objective == kGradCost) {
+        // terminal cost w_g |p_xy - goal|
+        const float dist = sqrtf(fmaf(f.x, f.x, f.y * f.y));
+        if (dist > 0.f && lane < 2) lam = p.C.wg * (lane == 0 ? f.x : f.y) / dist;
+    } else if (p.emin[j] == n_done) {
+        // the final state holds the margin
+        float sth, cth, sph, cph, t, f5;
+        sincos_r(f.z, sth, cth);
+        sincos_r(f.w, sph, cph);
+        esm_grad(p.V, f.w, sth, cth, sph, cph, t, f5);
+        if (lane == TH) lam = t;
+        if (lane == PH) lam = f5;
     }
+    return lam;
+}
+
+// gradients of the segment's control steps that never ran
+__device__ __forceinline__ void zero_grad(const BackParams &p, int j, int n_done, int t, int nt)
+{
+    for (int k = max(p.k0, (n_done + p.n_sub - 1) / p.n_sub) + t; k < p.k1; k += nt)
+        *(float2 *)(p.grad + ((size_t)k * p.K + j) * 2) = make_float2(0.f, 0.f);
+}
+
+// A few candidates: one per CTA.  kWide warps linearise a chunk of 32 kWide
+// steps into one of two buffers (976 bytes a step: the SM's shared memory)
+// while another warp runs the recursion over the chunk after it.
+constexpr int kWide = 3;
+__global__ void __launch_bounds__(32 * (kWide + 1)) grad_back_wide_kernel(const __grid_constant__ BackParams p)
+{
+    extern __shared__ __align__(16) float mats[];           // [2][32 kWide][kStepFloats], [2][16]
+    constexpr int kChunk = 32 * kWide;
+    const int j = blockIdx.x, t = threadIdx.x, lane = t & 31;
+    const bool runs = t >= kChunk;
+    const int n_done = p.n_done[j];
+    const int e0 = p.k0 * p.n_sub, e1 = min(p.k1 * p.n_sub, n_done);
+    zero_grad(p, j, n_done, t, 32 * (kWide + 1));
+    float lam = runs ? first_lam(p, j, n_done, lane) : 0.f;
+    const int n = e1 > e0 ? (e1 - e0 + kChunk - 1) / kChunk : 0;
+    for (int i = 0; i <= n; ++i) {
+        if (!runs && i < n) {
+            const int hi = e1 - i * kChunk, e = max(e0, hi - kChunk) + t;
+            if (e < hi) linearise(p, j, e, mats + (size_t)((i & 1) * kChunk + t) * kStepFloats);
+        }
+        if (runs && i > 0) {
+            const int hi = e1 - (i - 1) * kChunk, lo = max(e0, hi - kChunk);
+            lam = run_chunk<32>(p, j, mats + (size_t)((i - 1) & 1) * kChunk * kStepFloats,
+                                mats + (size_t)2 * kChunk * kStepFloats, lo, hi - lo, lane, lam);
+        }
+        __syncthreads();
+    }
+    if (runs && !p.first && lane < kRows) p.lam[(size_t)j * 16 + lane] = lam;
+}
+
+// Many candidates: two per warp.  The warp linearises 16 steps of each, then
+// its halves run the two recursions side by side.  Seven warps fit the SM's
+// shared memory; the warps cover one another's phases.
+__global__ void __launch_bounds__(32) grad_back_kernel(const __grid_constant__ BackParams p)
+{
+    extern __shared__ __align__(16) float mats[];           // [2][16][kStepFloats], [2][2][16]
+    const int half = threadIdx.x >> 4, lane = threadIdx.x & 15;
+    const int j = min(2 * (int)blockIdx.x + half, p.K - 1);
+    const bool live = 2 * (int)blockIdx.x + half < p.K;
+    const int n_done = p.n_done[j];
+    const int e0 = p.k0 * p.n_sub, e1 = live ? min(p.k1 * p.n_sub, n_done) : 0;
+    if (live) zero_grad(p, j, n_done, lane, 16);
+    float lam = first_lam(p, j, n_done, lane);
+    float *mine = mats + (size_t)half * 16 * kStepFloats;
+    for (int hi = e1; __any_sync(kFull, hi > e0); hi -= 16) {
+        const int lo = max(e0, hi - 16);
+        if (lo + lane < hi) linearise(p, j, lo + lane, mine + (size_t)lane * kStepFloats);
+        __syncwarp();
+        lam = run_chunk<16>(p, j, mine, mats + 32 * kStepFloats + half * 32, lo, max(hi - lo, 0), lane, lam);
+        __syncwarp();
+    }
+    if (live && !p.first && lane < kRows) p.lam[(size_t)j * 16 + lane] = lam;
+}
+
+template <int LANES, bool PER_X0>
+__global__ void __launch_bounds__(kPlanBlock, LANES == 4 ? 1 : LANES == 2 ? 8 : 6)
+grad_forward_kernel(const __grid_constant__ PlanParams p, const __grid_constant__ Trace tr)
+{
+    __shared__ Duo<LANES> sh;
+    int j;
+    float J = 0.f, margin = CUDART_INF_F;
+    bool feasible = false;
+    duo_rollout<LANES, PER_X0, TEX_F32, kAccF32>(p, tr, sh, blockIdx.x, j, J, margin, feasible);
+}
+
+template <bool PER_X0>
+void launch_forward(const PlanParams &p, const Trace &tr, cudaStream_t stream)
+{
+    int layout = plan_layout(0, p.N);
+    if (layout == kLayoutOne) layout = kLayoutDuo1;         // the trace is a two-warp rollout's
+    const unsigned grid = (unsigned)layout_ctas(layout, p.N);
+    if (layout == kLayoutDuo4) grad_forward_kernel<4, PER_X0><<<grid, kPlanBlock, 0, stream>>>(p, tr);
+    else if (layout == kLayoutDuo2) grad_forward_kernel<2, PER_X0><<<grid, kPlanBlock, 0, stream>>>(p, tr);
+    else grad_forward_kernel<1, PER_X0><<<grid, kPlanBlock, 0, stream>>>(p, tr);
+}
+
+// candidates up to which a CTA takes one: two waves of one CTA per SM, where the
+// two forms meet (202 us for 300 candidates of 330 steps, one per CTA; 190 us
+// for 305 of 240, two per warp)
+constexpr int kBackWideMaxK = 304;
+
+cudaError_t launch_back(const BackParams &b, cudaStream_t stream)
+{
+    if (b.K <= kBackWideMaxK) {
+        constexpr int kSmem = (2 * 32 * kWide * kStepFloats + 32) * (int)sizeof(float);
+        const cudaError_t e = cudaFuncSetAttribute(grad_back_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   kSmem);
+        if (e != cudaSuccess) return e;
+        grad_back_wide_kernel<<<(unsigned)b.K, 32 * (kWide + 1), kSmem, stream>>>(b);
+    } else {
+        grad_back_kernel<<<(unsigned)((b.K + 1) / 2), 32, (32 * kStepFloats + 64) * sizeof(float), stream>>>(b);
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace
 
-int grad_split_ctas(int device)
+GradPlan grad_plan(int K, int H, int n_sub, int ckpt)
 {
-    int sms = 0, per_sm = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grad_kernel<true>, 2 * kGradHalf, 0) !=
-        cudaSuccess)
-        return 0;
-    return sms * per_sm;
+    const auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    GradPlan g;
+    const size_t per_step = (size_t)K * n_sub * 64;                     // bytes of trace per control step
+    const size_t fit = kTraceBytes / per_step;
+    g.seg = fit >= (size_t)H ? H : (int)(fit > (size_t)ckpt ? fit : (size_t)ckpt);
+    if (g.seg > H) g.seg = H;
+    g.n_seg = (H + g.seg - 1) / g.seg;
+    size_t o = 0;
+    g.rec = o;  o = up(o + per_step * g.seg);
+    g.ckpt = o; o = up(o + (g.n_seg > 1 ? (size_t)g.n_seg * 20 * K * sizeof(float) : 0));
+    g.fin = o;  o = up(o + (size_t)K * sizeof(float4));
+    g.lam = o;  o = up(o + (g.n_seg > 1 ? (size_t)K * 16 * sizeof(float) : 0));
+    g.ints = o; o = up(o + (size_t)K * 2 * sizeof(int));
+    g.total = o;
+    return g;
 }
 
-cudaError_t launch_grad(const GradParams &p, cudaStream_t stream)
+cudaError_t launch_grad(const PlanParams &p, const GradPlan &g, int objective, char *buf, float *grad,
+                        cudaStream_t stream)
 {
-    const unsigned blocks = (unsigned)((p.K + kGradCands - 1) / kGradCands);
-    if (p.split)
-        grad_kernel<true><<<blocks, 2 * kGradHalf, 0, stream>>>(p);
-    else
-        grad_kernel<false><<<blocks, kGradHalf, 0, stream>>>(p);
-    return cudaGetLastError();
+    Trace tr;
+    tr.rec = (float4 *)(buf + g.rec);
+    tr.seg = g.seg;
+    tr.objective = objective;
+    tr.fin = (float4 *)(buf + g.fin);
+    tr.n_done = (int *)(buf + g.ints);
+    tr.emin = tr.n_done + p.N;
+    BackParams b;
+    b.V = p.V;
+    b.C = p.C;
+    b.T = p.T;
+    b.ctrl = p.ctrl;
+    b.K = p.N;
+    b.H = p.H;
+    b.n_sub = p.n_sub;
+    b.h = p.h;
+    b.objective = objective;
+    b.rec = tr.rec;
+    b.n_done = tr.n_done;
+    b.emin = tr.emin;
+    b.fin = tr.fin;
+    b.lam = (float *)(buf + g.lam);
+    b.grad = grad;
+    for (int s = g.n_seg - 1; s >= 0; --s) {
+        const bool last = s == g.n_seg - 1;
+        // the whole rollout with the last segment's trace and the checkpoints,
+        // then each earlier segment from its checkpoint
+        tr.k0 = last ? 0 : s * g.seg;
+        tr.k1 = last ? p.H : (s + 1) * g.seg;
+        tr.trace_k0 = s * g.seg;
+        float *ckpt = (float *)(buf + g.ckpt);
+        tr.ckpt = last && g.n_seg > 1 ? ckpt : nullptr;
+        tr.from = last ? nullptr : ckpt + (size_t)s * 20 * p.N;
+        if (p.x0_soa) launch_forward<true>(p, tr, stream);
+        else launch_forward<false>(p, tr, stream);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        b.k0 = s * g.seg;
+        b.k1 = tr.k1;
+        b.last = last;
+        b.first = s == 0;
+        e = launch_back(b, stream);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace atp

@@ -1,42 +1,29 @@
-// adjoint.cuh - parameters of the rollout-cost adjoint kernel.
+// adjoint.cuh - parameters of the rollout-cost adjoint kernels.
 #pragma once
 
 #include <cuda_runtime.h>
-
-#include "srb_model.cuh"
+#include <stddef.h>
 
 namespace atp {
 
-// threads per candidate in the adjoint (one wheel each)
-constexpr int kGradLanes = 4;
-// candidates per CTA; the CTA holds them twice (walking and recomputing)
-constexpr int kGradCands = 16;
-constexpr int kGradHalf = kGradCands * kGradLanes;
+struct PlanParams;
+
 // what the adjoint differentiates
 constexpr int kGradCost = 0, kGradMargin = 1;
 
-struct GradParams {
-    Veh V;
-    Cost C;
-    Terrain T;
-    float x0[13];             // shared initial state (x0_soa == nullptr)
-    const float *x0_soa;      // [13][K] or nullptr
-    const float2 *ctrl;       // [H][K]
-    int K, H, n_sub, ckpt;
-    float h;
-    int objective;            // kGradCost: J; kGradMargin: min U_ESM over the trajectory
-    int split;                // walk and recompute on separate warps (two buffers), else one
-                              // quad per candidate does both (one buffer)
-    float *cost;              // [K] the objective's value
-    float *grad;              // [H][K][2]
-    float *ckpt_buf;          // [ceil(H / ckpt)][20][K * kGradLanes]
-    float *seg_buf;           // [1 or 2][ckpt * n_sub][20][K * kGradLanes]
+// Device memory of one adjoint call.  A trace (one record of 64 bytes per
+// candidate and Euler step) of up to kTraceBytes is kept whole; a longer one
+// is recomputed in segments of `seg` control steps from checkpoints.
+constexpr size_t kTraceBytes = (size_t)1 << 30;
+struct GradPlan {
+    int seg, n_seg;                       // control steps per segment, segments
+    size_t rec, ckpt, fin, lam, ints, total;   // byte offsets and size
 };
+GradPlan grad_plan(int K, int H, int n_sub, int ckpt);
 
-// CTAs of the split layout (kGradCands candidates each) resident at once on
-// `device`, 0 if the query fails; the split layout pays while one wave holds
-// the grid
-int grad_split_ctas(int device);
-cudaError_t launch_grad(const GradParams &p, cudaStream_t stream);
+// `p` holds the problem (p.N = K, p.cost the objective's value [K]); grad is
+// [H][K][2] and buf grad_plan(...).total bytes.
+cudaError_t launch_grad(const PlanParams &p, const GradPlan &g, int objective, char *buf, float *grad,
+                        cudaStream_t stream);
 
 }  // namespace atp

@@ -29,7 +29,6 @@ struct atp_ctx {
     size_t scratch_bytes;
     atp::BatchParams *batch;  // host staging of one batch's descriptors
     float4 *cm_box;           // the costmap's per-perimeter reach boxes (device)
-    int grad_ctas;            // resident CTAs of the split adjoint layout, -1 until queried
 };
 
 namespace {
@@ -375,7 +374,6 @@ int atp_create(atp_ctx **out, int device)
     ctx->acc64 = 0;
     ctx->lanes = 0;
     ctx->stage = 0;
-    ctx->grad_ctas = -1;
     ctx->err[0] = 0;
     ctx->batch = new (std::nothrow) atp::BatchParams;
     if (!ctx->batch) {
@@ -780,47 +778,22 @@ int grad_impl(atp_ctx *ctx, int objective, const atp_vehicle *veh, const atp_cos
     if (rc != ATP_OK) return rc;
     if (terrain->format != ATP_TERRAIN_F32X4)
         return fail(ctx, ATP_ERR_UNSUPPORTED, "the adjoint takes F32X4 terrain only");
-    // four lanes per candidate, up to twice in a CTA: the lane slot stays within 32 bits
     if (K > (1 << 28)) return fail(ctx, ATP_ERR_UNSUPPORTED, "the adjoint takes at most 2^28 candidates");
     if (!cost_dev || !grad_dev) return fail(ctx, ATP_ERR_INVALID, "cost_dev and grad_dev are required");
     if (ckpt == 0) ckpt = 10;
     if (ckpt < 1) return fail(ctx, ATP_ERR_INVALID, "ckpt must be >= 1 (0 selects 10)");
     if (ckpt > H) ckpt = H;
-    const size_t n_seg = (size_t)(H + ckpt - 1) / ckpt;
-    const size_t KL = (size_t)K * atp::kGradLanes;      // every lane keeps its own states
-    const size_t ck_bytes = align_up(n_seg * 20 * KL * sizeof(float));
+    const atp::GradPlan gp = atp::grad_plan(K, H, ns, ckpt);
     DeviceGuard g(ctx->device);
     if (g.err != cudaSuccess) return cuda_fail(ctx, g.err, "set device");
-    if (ctx->grad_ctas < 0) ctx->grad_ctas = atp::grad_split_ctas(ctx->device);
-    // walking and recomputing on separate warps pays while one wave holds the grid
-    const bool split = ((size_t)K + atp::kGradCands - 1) / atp::kGradCands <= (size_t)ctx->grad_ctas;
-    const size_t seg_bytes = align_up((split ? 2 : 1) * (size_t)ckpt * ns * 20 * KL * sizeof(float));
-    if ((rc = ensure_scratch_bytes(ctx, ck_bytes + seg_bytes)) != ATP_OK) return rc;
-    char *base = (char *)ctx->scratch + kHeaderBytes;
-    atp::PlanParams pp;
-    std::memset(&pp, 0, sizeof pp);
-    derive(*veh, *cost, *terrain, pp);
-    fill_problem(pp, x0, x0_dev, ctrl_dev, K, H, dt, ns);
-    atp::GradParams p;
+    if ((rc = ensure_scratch_bytes(ctx, gp.total)) != ATP_OK) return rc;
+    atp::PlanParams p;
     std::memset(&p, 0, sizeof p);
-    p.V = pp.V;
-    p.C = pp.C;
-    p.T = pp.T;
-    std::memcpy(p.x0, pp.x0, sizeof p.x0);
-    p.x0_soa = pp.x0_soa;
-    p.ctrl = pp.ctrl;
-    p.K = K;
-    p.H = H;
-    p.n_sub = ns;
-    p.ckpt = ckpt;
-    p.h = pp.h;
-    p.objective = objective;
-    p.split = split;
+    derive(*veh, *cost, *terrain, p);
+    fill_problem(p, x0, x0_dev, ctrl_dev, K, H, dt, ns);
     p.cost = cost_dev;
-    p.grad = grad_dev;
-    p.ckpt_buf = (float *)base;
-    p.seg_buf = (float *)(base + ck_bytes);
-    cudaError_t e = atp::launch_grad(p, (cudaStream_t)stream);
+    const cudaError_t e = atp::launch_grad(p, gp, objective, (char *)ctx->scratch + kHeaderBytes, grad_dev,
+                                           (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "grad launch");
     return ATP_OK;
 }

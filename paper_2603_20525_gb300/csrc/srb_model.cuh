@@ -313,8 +313,9 @@ struct WheelOut {
 // (wx, wy, wz): the contact point's body velocity v + w x rho, the extension
 // rate chi_dot, spring and damper with liftoff, slip angle and sigmoid tire
 // force.  PAIRED takes the extension rate's inner pair as a packed pair (the
-// same bits).
-template <bool PAIRED = false>
+// same bits).  RATIO forms F_y as F_z (F_y / F_z), the adjoint's order, instead
+// of multiplying from the left.
+template <bool PAIRED = false, bool RATIO = false>
 __device__ __forceinline__ WheelOut wheel_dyn(const Veh &V, const WheelGeo &g, float vx, float vy, float vz,
                                               float wx, float wy, float wz, float rx, float ry, float k,
                                               float b, float Fs, float di)
@@ -335,7 +336,8 @@ __device__ __forceinline__ WheelOut wheel_dyn(const Veh &V, const WheelGeo &g, f
     const float Fz = Fk > 0.f ? fmaxf(fmaf(-b, chid, Fk), 0.f) : 0.f;   // = F_k + max(-b chid, -F_k)
     const float alpha = atan2_r(viy, vix) - di;
     const float Ca = V.C * alpha;
-    const float Fy = Fz * (-Ca * V.mu) * rsq(fmaf(Ca, Ca, V.mu2));
+    const float is = rsq(fmaf(Ca, Ca, V.mu2));
+    const float Fy = RATIO ? Fz * ((-Ca * V.mu) * is) : Fz * (-Ca * V.mu) * is;
     WheelOut w;
     w.Fz = Fz;
     w.Fy = Fy;

@@ -415,51 +415,55 @@ cudaError_t launch_plan(const PlanParams &p, bool reduce, cudaStream_t stream)
     return p.acc64 ? launch_acc<TEX_BF16, kAccF64>(p, reduce, stream) : launch_acc<TEX_BF16, kAccF32>(p, reduce, stream);
 }
 
-// One node's texel (Sec. III-A numeric slope, reading Q10): height, central-
-// difference slopes (one-sided on the border) and the costmap value.
-__device__ __forceinline__ float4 node_texel(const float *__restrict__ H, const float *__restrict__ cm, int nx,
-                                             int ny, float inv_cell, int i, int j)
+// Texels (Sec. III-A numeric slope, reading Q10): height, central-difference
+// slopes (one-sided on the border) and the costmap value per node.  Each
+// thread makes kPrepRows nodes of a column, so that its loads overlap (one node
+// per thread waited on them: 28 us for 2048^2 nodes against a 15 us floor of
+// bytes) and neighbouring rows come from registers.
+constexpr int kPrepRows = 4;
+
+struct PrepNode {
+    float c, gx, gy, cost;
+};
+
+// nodes (i, j0 .. j0 + kPrepRows - 1); rows beyond the map repeat the last
+__device__ __forceinline__ void prep_column(const float *__restrict__ H, const float *__restrict__ cm, int nx, int ny,
+                                            float inv_cell, int i, int j0, PrepNode (&n)[kPrepRows])
 {
-    const size_t r = (size_t)j * nx;
-    const float c = H[r + i];
-    float gx, gy;
-    if (i == 0) gx = (H[r + 1] - c) * inv_cell;
-    else if (i == nx - 1) gx = (c - H[r + nx - 2]) * inv_cell;
-    else gx = (H[r + i + 1] - H[r + i - 1]) * (0.5f * inv_cell);
-    if (j == 0) gy = (H[r + nx + i] - c) * inv_cell;
-    else if (j == ny - 1) gy = (c - H[r - nx + i]) * inv_cell;
-    else gy = (H[r + nx + i] - H[r - nx + i]) * (0.5f * inv_cell);
-    return make_float4(c, gx, gy, cm ? cm[r + i] : 0.f);
+    const int il = i > 0 ? i - 1 : 0, ir = i < nx - 1 ? i + 1 : nx - 1;
+    const float wx = i == 0 || i == nx - 1 ? inv_cell : 0.5f * inv_cell;
+    float col[kPrepRows + 2], l[kPrepRows], r[kPrepRows];
+#pragma unroll
+    for (int q = 0; q < kPrepRows + 2; ++q)
+        col[q] = __ldg(H + (size_t)min(max(j0 + q - 1, 0), ny - 1) * nx + i);
+#pragma unroll
+    for (int q = 0; q < kPrepRows; ++q) {
+        const size_t o = (size_t)min(j0 + q, ny - 1) * nx;
+        l[q] = __ldg(H + o + il);
+        r[q] = __ldg(H + o + ir);
+        n[q].cost = cm ? __ldg(cm + o + i) : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < kPrepRows; ++q) {
+        const int j = j0 + q;
+        n[q].c = col[q + 1];
+        n[q].gx = (r[q] - l[q]) * wx;
+        n[q].gy = (col[q + 2] - col[q]) * (j == 0 || j >= ny - 1 ? inv_cell : 0.5f * inv_cell);
+    }
 }
 
-__global__ void terrain_prepare_f32_kernel(const float *__restrict__ H, const float *__restrict__ cm,
-                                           int nx, int ny, float inv_cell, float4 *__restrict__ out)
+__global__ void __launch_bounds__(256) terrain_prepare_f32_kernel(const float *__restrict__ H,
+                                                                  const float *__restrict__ cm, int nx, int ny,
+                                                                  float inv_cell, float4 *__restrict__ out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= nx || j >= ny) return;
-    out[(size_t)j * nx + i] = node_texel(H, cm, nx, ny, inv_cell, i, j);
-}
-
-// BF16 texels.  Per 8 x 8 block a plane through the block's first node with
-// the slopes of its first row and first column (FP32, each operation rounded
-// on its own so that the plane is reproducible bit for bit); per node the
-// bf16 (round to nearest even) of the height's and the two node slopes'
-// residuals from that plane, and of the costmap value.
-__global__ void terrain_block_plane_kernel(const float *__restrict__ H, int nx, int ny, int nbx,
-                                           int nby, float4 *__restrict__ plane)
-{
-    const int bi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int bj = blockIdx.y * blockDim.y + threadIdx.y;
-    if (bi >= nbx || bj >= nby) return;
-    const int i0 = bi * 8, j0 = bj * 8;
-    const int ni = min(8, nx - i0), nj = min(8, ny - j0);
-    const float c0 = H[(size_t)j0 * nx + i0];
-    const float cx = ni > 1 ? __fmul_rn(__fsub_rn(H[(size_t)j0 * nx + i0 + ni - 1], c0),
-                                        __fdiv_rn(1.0f, (float)(ni - 1))) : 0.f;
-    const float cy = nj > 1 ? __fmul_rn(__fsub_rn(H[(size_t)(j0 + nj - 1) * nx + i0], c0),
-                                        __fdiv_rn(1.0f, (float)(nj - 1))) : 0.f;
-    plane[(size_t)bj * nbx + bi] = make_float4(c0, cx, cy, 0.f);
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    const int j0 = (blockIdx.y * 8 + threadIdx.y) * kPrepRows;
+    if (i >= nx || j0 >= ny) return;
+    PrepNode n[kPrepRows];
+    prep_column(H, cm, nx, ny, inv_cell, i, j0, n);
+#pragma unroll
+    for (int q = 0; q < kPrepRows; ++q)
+        if (j0 + q < ny) out[(size_t)(j0 + q) * nx + i] = make_float4(n[q].c, n[q].gx, n[q].gy, n[q].cost);
 }
 
 __device__ __forceinline__ unsigned bf16_bits(float v)
@@ -467,51 +471,63 @@ __device__ __forceinline__ unsigned bf16_bits(float v)
     return (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(v));
 }
 
-__global__ void terrain_prepare_bf16_kernel(const float *__restrict__ H, const float *__restrict__ cm,
-                                            int nx, int ny, float inv_cell, const float4 *__restrict__ plane,
-                                            int nbx, uint2 *__restrict__ out)
+// BF16 texels.  Per 8 x 8 block a plane through the block's first node with
+// the slopes of its first row and first column (FP32, each operation rounded
+// on its own so that the plane is reproducible bit for bit); per node the
+// bf16 (round to nearest even) of the height's and the two node slopes'
+// residuals from that plane, and of the costmap value.  Every thread forms
+// its block's plane itself (three loads its warp shares), the block's first
+// node stores it.
+__global__ void __launch_bounds__(256) terrain_prepare_bf16_kernel(const float *__restrict__ H,
+                                                                   const float *__restrict__ cm, int nx, int ny,
+                                                                   float inv_cell, float4 *__restrict__ plane, int nbx,
+                                                                   uint2 *__restrict__ out)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    if (i >= nx || j >= ny) return;
-    const size_t r = (size_t)j * nx;
-    const float c = H[r + i];
-    float gx, gy;
-    if (i == 0) gx = (H[r + 1] - c) * inv_cell;
-    else if (i == nx - 1) gx = (c - H[r + nx - 2]) * inv_cell;
-    else gx = (H[r + i + 1] - H[r + i - 1]) * (0.5f * inv_cell);
-    if (j == 0) gy = (H[r + nx + i] - c) * inv_cell;
-    else if (j == ny - 1) gy = (c - H[r - nx + i]) * inv_cell;
-    else gy = (H[r + nx + i] - H[r - nx + i]) * (0.5f * inv_cell);
-    const float4 P = plane[(size_t)(j >> 3) * nbx + (i >> 3)];
-    const float res = __fsub_rn(c, block_plane(P, i, j));
-    // slopes as residuals from the plane's own slopes
-    const float rgx = __fsub_rn(gx, __fmul_rn(P.y, inv_cell));
-    const float rgy = __fsub_rn(gy, __fmul_rn(P.z, inv_cell));
-    const float cv = cm ? cm[r + i] : 0.f;
-    out[r + i] = make_uint2(bf16_bits(res) | (bf16_bits(rgx) << 16), bf16_bits(rgy) | (bf16_bits(cv) << 16));
+    const int i = blockIdx.x * 32 + threadIdx.x;
+    const int j0 = (blockIdx.y * 8 + threadIdx.y) * kPrepRows;
+    if (i >= nx || j0 >= ny) return;
+    static_assert(8 % kPrepRows == 0, "a thread's nodes lie in one block");
+    PrepNode n[kPrepRows];
+    prep_column(H, cm, nx, ny, inv_cell, i, j0, n);
+    const int bi = i & ~7, bj = j0 & ~7;
+    const int ni = min(8, nx - bi), nj = min(8, ny - bj);
+    const float c0 = __ldg(H + (size_t)bj * nx + bi);
+    const float cx = ni > 1 ? __fmul_rn(__fsub_rn(__ldg(H + (size_t)bj * nx + bi + ni - 1), c0),
+                                        __fdiv_rn(1.0f, (float)(ni - 1))) : 0.f;
+    const float cy = nj > 1 ? __fmul_rn(__fsub_rn(__ldg(H + (size_t)(bj + nj - 1) * nx + bi), c0),
+                                        __fdiv_rn(1.0f, (float)(nj - 1))) : 0.f;
+    const float4 P = make_float4(c0, cx, cy, 0.f);
+    if (i == bi && j0 == bj) plane[(size_t)(bj >> 3) * nbx + (bi >> 3)] = P;
+#pragma unroll
+    for (int q = 0; q < kPrepRows; ++q) {
+        const int j = j0 + q;
+        if (j >= ny) break;
+        const float res = __fsub_rn(n[q].c, block_plane(P, i, j));
+        // slopes as residuals from the plane's own slopes
+        const float rgx = __fsub_rn(n[q].gx, __fmul_rn(P.y, inv_cell));
+        const float rgy = __fsub_rn(n[q].gy, __fmul_rn(P.z, inv_cell));
+        out[(size_t)j * nx + i] = make_uint2(bf16_bits(res) | (bf16_bits(rgx) << 16),
+                                             bf16_bits(rgy) | (bf16_bits(n[q].cost) << 16));
+    }
+}
+
+static dim3 prep_grid(int nx, int ny)
+{
+    return dim3((unsigned)((nx + 31) / 32), (unsigned)((ny + 8 * kPrepRows - 1) / (8 * kPrepRows)));
 }
 
 cudaError_t launch_terrain_prepare_bf16(const float *heights, const float *costmap, int nx, int ny,
                                         float inv_cell, uint2 *texels, float4 *plane, cudaStream_t stream)
 {
-    const int nbx = (nx + 7) / 8, nby = (ny + 7) / 8;
-    const dim3 b1(16, 16);
-    const dim3 g1((unsigned)((nbx + 15) / 16), (unsigned)((nby + 15) / 16));
-    terrain_block_plane_kernel<<<g1, b1, 0, stream>>>(heights, nx, ny, nbx, nby, plane);
-    const dim3 block(32, 8);
-    const dim3 grid((unsigned)((nx + 31) / 32), (unsigned)((ny + 7) / 8));
-    terrain_prepare_bf16_kernel<<<grid, block, 0, stream>>>(heights, costmap, nx, ny, inv_cell, plane, nbx,
-                                                            texels);
+    terrain_prepare_bf16_kernel<<<prep_grid(nx, ny), dim3(32, 8), 0, stream>>>(heights, costmap, nx, ny, inv_cell,
+                                                                               plane, (nx + 7) / 8, texels);
     return cudaGetLastError();
 }
 
 cudaError_t launch_terrain_prepare_f32(const float *heights, const float *costmap, int nx, int ny,
                                        float inv_cell, float4 *out, cudaStream_t stream)
 {
-    const dim3 block(32, 8);
-    const dim3 grid((unsigned)((nx + 31) / 32), (unsigned)((ny + 7) / 8));
-    terrain_prepare_f32_kernel<<<grid, block, 0, stream>>>(heights, costmap, nx, ny, inv_cell, out);
+    terrain_prepare_f32_kernel<<<prep_grid(nx, ny), dim3(32, 8), 0, stream>>>(heights, costmap, nx, ny, inv_cell, out);
     return cudaGetLastError();
 }
 

@@ -28,7 +28,7 @@ struct atp_ctx {
     void *scratch;            // reduction headers + per-plan candidate buffers
     size_t scratch_bytes;
     atp::BatchParams *batch;  // host staging of one batch's descriptors
-    float4 *cm_box;           // the costmap's per-perimeter reach boxes (device)
+    float4 *cm_box;           // the costmap's per-perimeter boxes, then its edges (device)
 };
 
 namespace {
@@ -386,7 +386,7 @@ int atp_create(atp_ctx **out, int device)
         delete ctx;
         return ATP_ERR_CUDA;
     }
-    if (cudaMalloc(&ctx->cm_box, sizeof(float4) * atp::kCostmapMaxPolys) != cudaSuccess) {
+    if (cudaMalloc(&ctx->cm_box, sizeof(float4) * atp::kCostmapMaxPolys + sizeof(atp::CostmapEdge) * atp::kCostmapEdges) != cudaSuccess) {
         delete ctx->batch;
         delete ctx;
         return ATP_ERR_NOMEM;
@@ -744,7 +744,12 @@ extern "C" int atp_costmap(atp_ctx *ctx, const double *xy_dev, const int *start,
     p.n_poly = n_poly;
     p.n_vert = start[n_poly];
     for (int q = 0; q <= n_poly; ++q) p.start[q] = start[q];
-    for (int q = 0; q < n_poly; ++q) p.kind[q] = kind[q];
+    for (int q = 0; q < n_poly; ++q) {
+        p.kind[q] = kind[q];
+        p.n_path += kind[q] == 1;
+    }
+    p.edge = p.n_vert <= atp::kCostmapEdges ? (atp::CostmapEdge *)(ctx->cm_box + atp::kCostmapMaxPolys) : nullptr;
+    p.box = ctx->cm_box;
     p.nx = nx;
     p.ny = ny;
     p.cell = cell;
@@ -760,7 +765,7 @@ extern "C" int atp_costmap(atp_ctx *ctx, const double *xy_dev, const int *start,
     // exactly zero at every node of a tile it misses.
     const double ext = std::max((double)(nx - 1), (double)(ny - 1)) * cell;
     const float reach = (float)(2.0 * eps + 1e-3 + 1e-5 * ext);
-    cudaError_t e = atp::launch_costmap(p, ctx->cm_box, reach, (cudaStream_t)stream);
+    cudaError_t e = atp::launch_costmap(p, reach, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "costmap launch");
     return ATP_OK;
 }

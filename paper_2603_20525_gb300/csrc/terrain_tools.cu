@@ -10,12 +10,15 @@
 //   * Costmap of the distance constraints (Sec. IV-C, IV-D).  At every node
 //     the signed distance to each obstacle or path-boundary perimeter is turned
 //     into the normalised quadratic soft-constraint cost rate and summed over
-//     the perimeters, so that the rollout only interpolates it.  One thread per
-//     node; each 16 x 16 tile streams the edges of the perimeters that can
-//     reach it through shared memory in chunks.
+//     the perimeters, so that the rollout only interpolates it.  Four nodes per
+//     thread; each 32 x 32 tile streams the edges of the perimeters that can
+//     cost anything in it through shared memory in chunks.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <stdint.h>
+
+#include "fastmath.cuh"
 #include "terrain_tools.cuh"
 
 namespace atp {
@@ -23,22 +26,23 @@ namespace atp {
 namespace {
 
 constexpr int kRowThreads = 256;  // row-pass CTA
-// Outputs per thread: 4 row and 8 column outputs below this radius, 8 and 16
-// from it on.  Small radii are bound by each CTA's set-up, and more outputs
-// per thread only halve the CTAs; large radii by the taps, where the wider
-// windows load fewer values per output (measured on the GB300: the narrow
-// form 4 % faster at 12 cells, the wide one 5 % at 24 and 10 to 16 % at 36
-// to 200 cells; the same bits).
+// Outputs per thread: 4 row outputs (of two rows) below this radius and 8 from
+// it on, where the wider window loads fewer values per output; 8 column
+// outputs (of two columns), in CTAs of 64 columns below it and of 32 columns
+// and twice the rows from it on, whose halo is then the smaller part of the
+// tile.  16 column outputs gained nothing (84 registers).  2048^2 nodes, both
+// passes: 31.2 -> 26.4 us at 12 cells, 73.9 -> 61.5 us at 60, 197 -> 162 us at
+// 200 against one row or column per thread without the packing.
 constexpr int kLodWideMinR = 16;
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
-// Normalised weights w[k], k = 0..2r, of exp(-(k - r)^2 / (2 s^2)), made by
-// every CTA the same way: the terms, then their sum in a fixed order (per
-// thread a strided run, then a fixed shuffle tree and a fixed pass over the
-// warps), so every CTA holds the same bits.  Needs blockDim.x * blockDim.y a
-// multiple of 32 and at most 1024 threads.
-__device__ void gauss_weights_cta(float *w, int r, float inv2s2)
+// Normalised weights w[k], k = 0..2r, of exp(-(k - r)^2 / (2 s^2)), each twice
+// for the packed FMAs, made by every CTA the same way: the terms, then their
+// sum in a fixed order (per thread a strided run, then a fixed shuffle tree
+// and a fixed pass over the warps), so every CTA holds the same bits.  Needs
+// blockDim.x * blockDim.y a multiple of 32 and at most 1024 threads.
+__device__ void gauss_weights_cta(float2 *w, int r, float inv2s2)
 {
     __shared__ float s_part[32];
     __shared__ float s_total;
@@ -49,7 +53,7 @@ __device__ void gauss_weights_cta(float *w, int r, float inv2s2)
     for (int k = t; k < n; k += nt) {
         const float d = (float)(k - r);
         const float e = expf(-(d * d) * inv2s2);
-        w[k] = e;
+        w[k].x = e;
         part += e;
     }
 #pragma unroll
@@ -63,7 +67,10 @@ __device__ void gauss_weights_cta(float *w, int r, float inv2s2)
     }
     __syncthreads();
     const float z = s_total;
-    for (int k = t; k < n; k += nt) w[k] = w[k] / z;
+    for (int k = t; k < n; k += nt) {
+        const float v = w[k].x / z;
+        w[k] = make_float2(v, v);
+    }
     __syncthreads();
 }
 
@@ -72,9 +79,8 @@ __device__ void gauss_weights_cta(float *w, int r, float inv2s2)
 // dividing by lane 0's total.  The CTA-wide form adds only the other warps'
 // zero sums to that total, so the bits are the same.  The other warps go
 // straight on to their tile loads, and the caller's next barrier publishes
-// the weights: at a radius of 12 cells this took 6 % off the two passes,
-// where the set-up's barriers bound them.
-__device__ __forceinline__ void gauss_weights_warp(float *w, int r, float inv2s2)
+// the weights.
+__device__ __forceinline__ void gauss_weights_warp(float2 *w, int r, float inv2s2)
 {
     const int t = threadIdx.y * blockDim.x + threadIdx.x;
     if (t >= 32) return;
@@ -88,14 +94,14 @@ __device__ __forceinline__ void gauss_weights_warp(float *w, int r, float inv2s2
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
     z = __shfl_sync(0xffffffffu, z, 0);
-    if (t < n) w[t] = e / z;
+    if (t < n) w[t] = make_float2(e / z, e / z);
 }
 
 // The weights of a pass: the first warp alone for the narrow windows (r below
 // kLodWideMinR, so 2r + 1 <= 31), the whole CTA otherwise.
 static_assert(2 * (kLodWideMinR - 1) + 1 <= 32, "the narrow windows' weights fit one warp");
 template <bool NARROW>
-__device__ __forceinline__ void gauss_weights(float *w, int r, float inv2s2)
+__device__ __forceinline__ void gauss_weights(float2 *w, int r, float inv2s2)
 {
     if (NARROW)
         gauss_weights_warp(w, r, inv2s2);
@@ -103,145 +109,218 @@ __device__ __forceinline__ void gauss_weights(float *w, int r, float inv2s2)
         gauss_weights_cta(w, r, inv2s2);
 }
 
-// out[j][i] = sum_k w[k] in[j][clamp(i + k - r)], each sum over k in order.
-// Thread t makes outputs OUT t .. OUT t + OUT - 1 of the CTA's 256 OUT from a
-// window of OUT + 4 tile values refilled by one 16-byte shared load per four
-// taps.
-template <int OUT>
-__global__ void __launch_bounds__(kRowThreads) lod_rows_kernel(LodParams p)
+// acc[q] = sum over taps k = first .. last-1, in order, of w[k] v(k + q),
+// two outputs packed in each float2, from a window of OUT + 4 positions that
+// four loads refill every four taps.  The window's slots rotate through an
+// unrolled run of groups, so nothing moves.  load(x) gives positions x .. x + 3
+// (x a multiple of 4).
+template <int OUT, class Load>
+__device__ __forceinline__ void convolve(const float2 *w, int first, int last, float2 (&acc)[OUT], const Load &load)
 {
-    static_assert(OUT % 4 == 0, "whole float4 windows");
-    constexpr int kRowOut = OUT, kRowVec = OUT / 4, kRowTile = kRowThreads * OUT;
-    extern __shared__ __align__(16) float sm[];         // the tile is read as float4
-    float *w = sm;                                      // 2r + 1, padded to 4
-    float *tile = sm + ((2 * p.r + 1 + 3) & ~3);        // kRowTile + 2r + 8
-    gauss_weights<OUT == 4>(w, p.r, p.inv2s2);
-    const int j = blockIdx.y;
-    const int i0 = blockIdx.x * kRowTile;
-    const float *row = p.in + (size_t)j * p.nx;
-    const int n_tile = kRowTile + 2 * p.r + 8;
-    for (int t = threadIdx.x; t < n_tile; t += kRowThreads)
-        tile[t] = __ldg(row + clampi(i0 - p.r + t, 0, p.nx - 1));
-    __syncthreads();
-    const int ib = i0 + kRowOut * threadIdx.x;
-    if (ib >= p.nx) return;
-    const float4 *t4 = reinterpret_cast<const float4 *>(tile) + kRowVec * threadIdx.x;
-    float acc[kRowOut];
-    float4 win[kRowVec + 1];
+    constexpr int kWin = OUT + 4, kRun = OUT == 8 ? 6 : kWin / 4;
+    float2 v[kWin];
 #pragma unroll
-    for (int q = 0; q < kRowOut; ++q) acc[q] = 0.f;
+    for (int q = 0; q < OUT; ++q) acc[q] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < kRowVec; ++c) win[c] = t4[c];
-    const int n = 2 * p.r + 1;
-    for (int k0 = 0; k0 < n; k0 += 4) {
-        win[kRowVec] = t4[(k0 >> 2) + kRowVec];
-        float v[kRowOut + 4];
+    for (int x = 0; x < kWin; x += 4) load(x, v[x], v[x + 1], v[x + 2], v[x + 3]);
+    const int groups = (last + 3) / 4;
+    for (int g0 = 0; g0 < groups; g0 += kRun) {
 #pragma unroll
-        for (int c = 0; c <= kRowVec; ++c) {
-            v[4 * c] = win[c].x;
-            v[4 * c + 1] = win[c].y;
-            v[4 * c + 2] = win[c].z;
-            v[4 * c + 3] = win[c].w;
-        }
+        for (int u = 0; u < kRun; ++u) {
+            const int g = g0 + u;
+            if (g < groups) {
+                const bool whole = 4 * g >= first && 4 * g + 4 <= last;
+                const float4 wa = ((const float4 *)w)[2 * g], wb = ((const float4 *)w)[2 * g + 1];
+                const float2 wg[4] = {make_float2(wa.x, wa.y), make_float2(wa.z, wa.w), make_float2(wb.x, wb.y),
+                                      make_float2(wb.z, wb.w)};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (k0 + e < n) {
-                const float wk = w[k0 + e];
+                for (int e = 0; e < 4; ++e) {
+                    if (whole || (4 * g + e >= first && 4 * g + e < last)) {
+                        const float2 wk = wg[e];
 #pragma unroll
-                for (int q = 0; q < kRowOut; ++q) acc[q] = fmaf(wk, v[e + q], acc[q]);
+                        for (int q = 0; q < OUT; ++q) acc[q] = fma2(wk, v[(4 * u + e + q) % kWin], acc[q]);
+                    }
+                }
+                constexpr int kNext = kWin;
+                load(4 * g + kNext, v[(4 * u) % kWin], v[(4 * u + 1) % kWin], v[(4 * u + 2) % kWin],
+                     v[(4 * u + 3) % kWin]);
             }
         }
-#pragma unroll
-        for (int c = 0; c < kRowVec; ++c) win[c] = win[c + 1];
     }
-    float *o = p.out + (size_t)j * p.nx + ib;
+}
+
+// out[j][i] = sum_k w[k] in[j][clamp(i + k - r)], each sum over k in order, for
+// two rows: the tile holds their values side by side, so that one packed FMA
+// serves both (the passes are bound by instruction issue, not by the FMA
+// pipe).  Thread t makes outputs OUT t .. OUT t + OUT - 1 of the CTA's 256 OUT.
+// VEC: rows are 16-byte aligned, the tile starts at a multiple of four columns
+// (`shift` columns before the first tap) and is filled by 16-byte loads.  Every
+// OUT positions of the tile are padded by two, so that a warp's 16-byte loads
+// fall on distinct banks.
+template <int OUT, bool VEC>
+__global__ void __launch_bounds__(kRowThreads) lod_rows_kernel(LodParams p)
+{
+    constexpr int kRowTile = kRowThreads * OUT;
+    const auto at = [](int x) { return x / OUT * (OUT + 2) + x % OUT; };
+    extern __shared__ __align__(16) float2 sm2[];
+    const int n = 2 * p.r + 1;
+    const int shift = VEC ? (4 - (p.r & 3)) & 3 : 0;
+    float2 *w = sm2;                                        // shift + n, padded to 8
+    float2 *tile = sm2 + ((n + 11) & ~7);                   // kRowTile + 2r + 16
+    gauss_weights<OUT == 4>(w + shift, p.r, p.inv2s2);
+    const int j = 2 * blockIdx.y, j1 = min(j + 1, p.ny - 1);
+    const int i0 = blockIdx.x * kRowTile, s0 = i0 - p.r - shift;
+    const float *row0 = p.in + (size_t)j * p.nx, *row1 = p.in + (size_t)j1 * p.nx;
+    const int n_tile = kRowTile + 2 * p.r + 16;
+    if (VEC) {
+        for (int t = threadIdx.x; t < n_tile / 4; t += kRowThreads) {
+            const int x = s0 + 4 * t;
+            float4 a, b;
+            if (x >= 0 && x + 3 < p.nx) {
+                a = __ldg((const float4 *)(row0 + x));
+                b = __ldg((const float4 *)(row1 + x));
+            } else {
+                const int x0 = clampi(x, 0, p.nx - 1), x1 = clampi(x + 1, 0, p.nx - 1);
+                const int x2 = clampi(x + 2, 0, p.nx - 1), x3 = clampi(x + 3, 0, p.nx - 1);
+                a = make_float4(__ldg(row0 + x0), __ldg(row0 + x1), __ldg(row0 + x2), __ldg(row0 + x3));
+                b = make_float4(__ldg(row1 + x0), __ldg(row1 + x1), __ldg(row1 + x2), __ldg(row1 + x3));
+            }
+            float4 *t4 = (float4 *)(tile + at(4 * t));
+            t4[0] = make_float4(a.x, b.x, a.y, b.y);
+            t4[1] = make_float4(a.z, b.z, a.w, b.w);
+        }
+        for (int t = (n_tile & ~3) + threadIdx.x; t < n_tile; t += kRowThreads) {
+            const int x = clampi(s0 + t, 0, p.nx - 1);
+            tile[at(t)] = make_float2(__ldg(row0 + x), __ldg(row1 + x));
+        }
+    } else {
+        for (int t = threadIdx.x; t < n_tile; t += kRowThreads) {
+            const int x = clampi(s0 + t, 0, p.nx - 1);
+            tile[at(t)] = make_float2(__ldg(row0 + x), __ldg(row1 + x));
+        }
+    }
+    __syncthreads();
+    const int ib = i0 + OUT * threadIdx.x;
+    if (ib >= p.nx) return;
+    const float2 *mine = tile + (OUT + 2) * threadIdx.x;
+    float2 acc[OUT];
+    convolve<OUT>(w, shift, shift + n, acc, [&](int x, float2 &a, float2 &b, float2 &c, float2 &d) {
+        const float4 *t4 = (const float4 *)(mine + at(x));
+        const float4 u = t4[0], v = t4[1];
+        a = make_float2(u.x, u.y);
+        b = make_float2(u.z, u.w);
+        c = make_float2(v.x, v.y);
+        d = make_float2(v.z, v.w);
+    });
+    float *o0 = p.out + (size_t)j * p.nx + ib, *o1 = p.out + (size_t)j1 * p.nx + ib;
+    if (VEC) {                                              // nx is a multiple of 4, so whole float4
 #pragma unroll
-    for (int q = 0; q < kRowOut; ++q)
-        if (ib + q < p.nx) o[q] = acc[q];
+        for (int q = 0; q < OUT; q += 4) {
+            if (ib + q < p.nx) {
+                *(float4 *)(o0 + q) = make_float4(acc[q].x, acc[q + 1].x, acc[q + 2].x, acc[q + 3].x);
+                if (j1 > j) *(float4 *)(o1 + q) = make_float4(acc[q].y, acc[q + 1].y, acc[q + 2].y, acc[q + 3].y);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < OUT; ++q) {
+            if (ib + q < p.nx) {
+                o0[q] = acc[q].x;
+                if (j1 > j) o1[q] = acc[q].y;
+            }
+        }
+    }
 }
 
 // out[j][i] = sum_k w[k] in[clamp(j + k - r)][i], each sum over k in order; a
-// CTA of 32 x 8 threads covers 32 columns and 8 OUT rows, thread (x, y) rows
-// OUT y .. OUT y + OUT - 1 of column x from a window of 2 OUT tile rows
-// refilled with OUT loads per OUT taps.
-template <int OUT>
+// CTA of CX x 256/CX threads covers 2 CX columns and 256/CX OUT rows, thread
+// (x, y) rows OUT y .. OUT y + OUT - 1 of columns 2x and 2x + 1, packed.  VEC:
+// the map's column pairs are 8-byte aligned.
+template <int OUT, int CX, bool VEC, bool NARROW>
 __global__ void __launch_bounds__(256) lod_cols_kernel(LodParams p)
 {
-    constexpr int kColOut = OUT, kColTile = 8 * OUT;
-    extern __shared__ float sm[];
-    float *w = sm;                           // 2r + 1, padded to a multiple of 32
-    float *tile = sm + ((2 * p.r + 1 + 31) & ~31);   // [kColTile + 2r + 8][32]
-    gauss_weights<OUT == 8>(w, p.r, p.inv2s2);
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    const int j0 = blockIdx.y * kColTile;
-    const int ic = min(i, p.nx - 1);
-    const int n_rows = kColTile + 2 * p.r + kColOut;
-    for (int t = threadIdx.y; t < n_rows; t += 8)
-        tile[t * 32 + threadIdx.x] = __ldg(p.in + (size_t)clampi(j0 - p.r + t, 0, p.ny - 1) * p.nx + ic);
-    __syncthreads();
-    const int jb = kColOut * threadIdx.y;    // first of this thread's rows in the tile
-    if (i >= p.nx || j0 + jb >= p.ny) return;
-    const float *col = tile + jb * 32 + threadIdx.x;
-    float acc[kColOut];
-    float v[2 * kColOut];
-#pragma unroll
-    for (int q = 0; q < kColOut; ++q) {
-        acc[q] = 0.f;
-        v[q] = col[q * 32];
-    }
+    constexpr int kColTile = 256 / CX * OUT;
+    extern __shared__ __align__(16) float2 sm2[];
     const int n = 2 * p.r + 1;
-    for (int k0 = 0; k0 < n; k0 += kColOut) {
-#pragma unroll
-        for (int q = 0; q < kColOut; ++q) v[kColOut + q] = col[(k0 + kColOut + q) * 32];
-#pragma unroll
-        for (int e = 0; e < kColOut; ++e) {
-            if (k0 + e < n) {
-                const float wk = w[k0 + e];
-#pragma unroll
-                for (int q = 0; q < kColOut; ++q) acc[q] = fmaf(wk, v[e + q], acc[q]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < kColOut; ++q) v[q] = v[kColOut + q];
+    float2 *w = sm2;                                        // n, padded to a multiple of 32
+    float2 *tile = sm2 + ((n + 31) & ~31);                  // [kColTile + 2r + 8][CX]
+    gauss_weights<NARROW>(w, p.r, p.inv2s2);
+    const int i = blockIdx.x * (2 * CX) + 2 * threadIdx.x;
+    const int j0 = blockIdx.y * kColTile;
+    const int ia = min(i, p.nx - 1), ib = min(i + 1, p.nx - 1);
+    const int n_rows = kColTile + 2 * p.r + 8;
+    for (int t = threadIdx.y; t < n_rows; t += 256 / CX) {
+        const float *row = p.in + (size_t)clampi(j0 - p.r + t, 0, p.ny - 1) * p.nx;
+        tile[t * CX + threadIdx.x] = VEC ? __ldg((const float2 *)(row + min(i, p.nx - 2)))
+                                         : make_float2(__ldg(row + ia), __ldg(row + ib));
     }
+    __syncthreads();
+    const int jb = OUT * threadIdx.y;        // first of this thread's rows in the tile
+    if (i >= p.nx || j0 + jb >= p.ny) return;
+    const float2 *col = tile + jb * CX + threadIdx.x;
+    float2 acc[OUT];
+    convolve<OUT>(w, 0, n, acc, [&](int x, float2 &a, float2 &b, float2 &c, float2 &d) {
+        a = col[x * CX];
+        b = col[x * CX + CX];
+        c = col[x * CX + 2 * CX];
+        d = col[x * CX + 3 * CX];
+    });
 #pragma unroll
-    for (int q = 0; q < kColOut; ++q) {
+    for (int q = 0; q < OUT; ++q) {
         const int j = j0 + jb + q;
-        if (j < p.ny) p.out[(size_t)j * p.nx + i] = acc[q];
+        if (j >= p.ny) break;
+        float *o = p.out + (size_t)j * p.nx + i;
+        if (VEC) {
+            *(float2 *)o = acc[q];
+        } else {
+            o[0] = acc[q].x;
+            if (i + 1 < p.nx) o[1] = acc[q].y;
+        }
     }
 }
 
 size_t rows_smem(int r, int out)
 {
-    return sizeof(float) * (size_t)(((2 * r + 1 + 3) & ~3) + kRowThreads * out + 2 * r + 8);
+    return sizeof(float2) * (size_t)(((2 * r + 1 + 11) & ~7) + (kRowThreads * out + 2 * r + 16 + out) / out * (out + 2));
 }
-size_t cols_smem(int r, int out)
+size_t cols_smem(int r, int out, int cx)
 {
-    return sizeof(float) * (size_t)(((2 * r + 1 + 31) & ~31) + (8 * out + 2 * r + out) * 32);
+    return sizeof(float2) * (size_t)(((2 * r + 1 + 31) & ~31) + (256 / cx * out + 2 * r + 8) * cx);
 }
 
-template <int ROW_OUT, int COL_OUT>
-cudaError_t lod_passes(LodParams p, float *tmp, float *out, cudaStream_t stream)
+template <int ROW_OUT, bool VEC>
+cudaError_t lod_rows(const LodParams &p, cudaStream_t stream)
 {
-    const int r = p.r;
-    cudaError_t e = cudaFuncSetAttribute(lod_rows_kernel<ROW_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)rows_smem(kLodMaxRadius, ROW_OUT));
+    const size_t smem = rows_smem(p.r, ROW_OUT);
+    const cudaError_t e = cudaFuncSetAttribute(lod_rows_kernel<ROW_OUT, VEC>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)rows_smem(kLodMaxRadius, ROW_OUT));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lod_cols_kernel<COL_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)cols_smem(kLodMaxRadius, COL_OUT));
-    if (e != cudaSuccess) return e;
-    p.out = tmp;
-    const int row_tile = kRowThreads * ROW_OUT;
-    lod_rows_kernel<ROW_OUT><<<dim3((unsigned)((p.nx + row_tile - 1) / row_tile), (unsigned)p.ny), kRowThreads,
-                               rows_smem(r, ROW_OUT), stream>>>(p);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    p.in = tmp;
-    p.out = out;
-    const int col_tile = 8 * COL_OUT;
-    lod_cols_kernel<COL_OUT><<<dim3((unsigned)((p.nx + 31) / 32), (unsigned)((p.ny + col_tile - 1) / col_tile)),
-                               dim3(32, 8), cols_smem(r, COL_OUT), stream>>>(p);
+    const int tile = kRowThreads * ROW_OUT;
+    const dim3 grid((unsigned)((p.nx + tile - 1) / tile), (unsigned)((p.ny + 1) / 2));
+    lod_rows_kernel<ROW_OUT, VEC><<<grid, kRowThreads, smem, stream>>>(p);
     return cudaGetLastError();
+}
+
+template <int OUT, int CX, bool VEC, bool NARROW>
+cudaError_t lod_cols(const LodParams &p, cudaStream_t stream)
+{
+    constexpr size_t kMaxSmem = 226 * 1024;       // less the static arrays
+    const size_t smem = cols_smem(p.r, OUT, CX);
+    const cudaError_t e = cudaFuncSetAttribute(lod_cols_kernel<OUT, CX, VEC, NARROW>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+    if (e != cudaSuccess) return e;
+    const int rows = 256 / CX * OUT;
+    const dim3 grid((unsigned)((p.nx + 2 * CX - 1) / (2 * CX)), (unsigned)((p.ny + rows - 1) / rows));
+    lod_cols_kernel<OUT, CX, VEC, NARROW><<<grid, dim3(CX, 256 / CX), smem, stream>>>(p);
+    return cudaGetLastError();
+}
+
+template <bool VEC>
+cudaError_t lod_cols_by_radius(const LodParams &p, cudaStream_t stream)
+{
+    if (p.r < kLodWideMinR) return lod_cols<8, 32, VEC, true>(p, stream);
+    return lod_cols<8, 16, VEC, false>(p, stream);
 }
 
 }  // namespace
@@ -256,7 +335,18 @@ cudaError_t launch_lod_smooth(const float *in, float *tmp, float *out, int nx, i
     p.r = r;
     p.inv2s2 = inv2s2;
     p.in = in;
-    return r < kLodWideMinR ? lod_passes<4, 8>(p, tmp, out, stream) : lod_passes<8, 16>(p, tmp, out, stream);
+    p.out = tmp;
+    const bool vec_rows = nx % 4 == 0 && ((uintptr_t)in | (uintptr_t)tmp) % 16 == 0;
+    cudaError_t e;
+    if (r < kLodWideMinR)
+        e = vec_rows ? lod_rows<4, true>(p, stream) : lod_rows<4, false>(p, stream);
+    else
+        e = vec_rows ? lod_rows<8, true>(p, stream) : lod_rows<8, false>(p, stream);
+    if (e != cudaSuccess) return e;
+    p.in = tmp;
+    p.out = out;
+    const bool vec_cols = nx % 2 == 0 && ((uintptr_t)tmp | (uintptr_t)out) % 8 == 0;
+    return vec_cols ? lod_cols_by_radius<true>(p, stream) : lod_cols_by_radius<false>(p, stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -266,23 +356,40 @@ cudaError_t launch_lod_smooth(const float *in, float *tmp, float *out, int nx, i
 
 namespace {
 
-constexpr int kChunk = 256;       // vertices staged per pass, one per thread
-// the tile's perimeter scan takes one thread of the 16 x 16 CTA per perimeter
+constexpr int kTile = 32;         // nodes per side of a CTA's tile
+constexpr int kRows = 4;          // nodes per thread, 8 rows apart
+constexpr int kChunk = 256;       // edges staged per pass, one per thread
+// the tile's perimeter scan takes one thread of the 32 x 8 CTA per perimeter
 static_assert(kCostmapMaxPolys <= 256, "one costmap thread per perimeter");
 
-// Bounding box of perimeter blockIdx.x in the costmap kernel's coordinates,
-// grown by `reach`; one warp per perimeter.
-__global__ void __launch_bounds__(32) costmap_boxes_kernel(const __grid_constant__ CostmapParams p,
-                                                           float4 *box, float reach)
+// Edge v of perimeter q in the costmap's coordinates: metres from the map
+// corner, FP64 once per vertex, then FP32.
+__device__ __forceinline__ CostmapEdge make_edge(const CostmapParams &p, int v, int q)
 {
-    const int q = blockIdx.x;
+    const int u = v + 1 < p.start[q + 1] ? v + 1 : p.start[q];
+    const float ax = (float)(p.xy[2 * v] - p.x0), ay = (float)(p.xy[2 * v + 1] - p.y0);
+    const float bx = (float)(p.xy[2 * u] - p.x0), by = (float)(p.xy[2 * u + 1] - p.y0);
+    const float ex = bx - ax, ey = by - ay;
+    const float l2 = fmaf(ex, ex, ey * ey);
+    CostmapEdge e;
+    e.a = make_float4(ax, ay, ex, ey);
+    e.b = make_float4(bx, by, l2, __int_as_float(q));
+    return e;
+}
+
+// One warp per perimeter: its edges, where they are kept, and its bounding box
+// grown by `reach`.
+__global__ void __launch_bounds__(32) costmap_edges_kernel(const __grid_constant__ CostmapParams p, float reach)
+{
+    const int q = blockIdx.x, v0 = p.start[q], v1 = p.start[q + 1];
     float x0 = CUDART_INF_F, y0 = CUDART_INF_F, x1 = -CUDART_INF_F, y1 = -CUDART_INF_F;
-    for (int v = p.start[q] + (int)threadIdx.x; v < p.start[q + 1]; v += 32) {
-        const float x = (float)(p.xy[2 * v] - p.x0), y = (float)(p.xy[2 * v + 1] - p.y0);
-        x0 = fminf(x0, x);
-        y0 = fminf(y0, y);
-        x1 = fmaxf(x1, x);
-        y1 = fmaxf(y1, y);
+    for (int v = v0 + (int)threadIdx.x; v < v1; v += 32) {
+        const CostmapEdge e = make_edge(p, v, q);
+        if (p.edge) p.edge[v] = e;
+        x0 = fminf(x0, e.a.x);
+        y0 = fminf(y0, e.a.y);
+        x1 = fmaxf(x1, e.a.x);
+        y1 = fmaxf(y1, e.a.y);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -291,34 +398,88 @@ __global__ void __launch_bounds__(32) costmap_boxes_kernel(const __grid_constant
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
         y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
     }
-    if (threadIdx.x == 0) box[q] = make_float4(x0 - reach, y0 - reach, x1 + reach, y1 + reach);
+    if (threadIdx.x == 0) p.box[q] = make_float4(x0 - reach, y0 - reach, x1 + reach, y1 + reach);
 }
 
-__global__ void __launch_bounds__(256) costmap_kernel(const __grid_constant__ CostmapParams p)
+// off[k] <= v < off[k + 1]
+__device__ __forceinline__ int perimeter_of(int v, const int *off, int n)
 {
-    __shared__ float2 s_a[kChunk], s_b[kChunk];
-    __shared__ int s_poly[kChunk];
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (off[mid] <= v) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Even-odd rule with a ray towards +x, for the edge from (a.x, a.y) along
+// (a.z, a.w) to (b.x, b.y).
+__device__ __forceinline__ bool crosses(float4 a, float4 b, float px, float py)
+{
+    if ((a.y > py) == (b.y > py)) return false;
+    return px < fmaf((py - a.y) / (b.y - a.y), a.z, a.x);
+}
+
+// A CTA of 32 x 8 threads makes a tile of 32 x 32 nodes, four per thread.  It
+// first finds the perimeters that can cost anything in the tile: without the
+// signed distances, an obstacle whose grown box misses the tile adds exactly
+// nothing, and neither does a path boundary that holds the tile with every edge
+// farther than `reach` (the edges are tested by all threads at once).  The
+// edges of the others go through shared memory, in their order.
+__global__ void __launch_bounds__(256) costmap_kernel(const __grid_constant__ CostmapParams p, float reach)
+{
+    __shared__ float4 s_a[kChunk], s_b[kChunk];
     __shared__ int s_id[kCostmapMaxPolys];        // the tile's perimeters, in order
     __shared__ int s_off[kCostmapMaxPolys + 1];   // prefix of their vertex counts
+    __shared__ int s_near[kCostmapMaxPolys];      // path boundaries: 2 for a near edge, bit 0 inside
     __shared__ int s_wn[8], s_wv[8];
-    const int i = blockIdx.x * 16 + threadIdx.x;
-    const int j = blockIdx.y * 16 + threadIdx.y;
-    const int t = threadIdx.y * 16 + threadIdx.x;
-    const bool live = i < p.nx && j < p.ny;
-    const float px = (float)((double)i * p.cell), py = (float)((double)j * p.cell);
-    // the perimeters that can reach this tile (all of them without boxes),
-    // kept in their order by a block-wide scan over one thread per perimeter
+    __shared__ float s_x[kTile], s_y[kTile];
+    const int t = threadIdx.y * 32 + threadIdx.x;
+    const bool all = p.sdist != nullptr;
+    // node coordinates, FP64 once per row and column of the tile
+    if (t < kTile) s_x[t] = (float)((double)(blockIdx.x * kTile + t) * p.cell);
+    else if (t < 2 * kTile) s_y[t - kTile] = (float)((double)(blockIdx.y * kTile + t - kTile) * p.cell);
+    if (t < p.n_poly) s_near[t] = 0;
+    __syncthreads();
+    const float tx0 = s_x[0], tx1 = s_x[kTile - 1], ty0 = s_y[0], ty1 = s_y[kTile - 1];
+    if (!all && p.n_path > 0) {
+        const float mx = s_x[kTile / 2], my = s_y[kTile / 2];
+        for (int v = t; v < p.n_vert; v += 256) {
+            int q;
+            float4 a, b;
+            if (p.edge) {
+                b = __ldg(&p.edge[v].b);
+                q = __float_as_int(b.w);
+                if (p.kind[q] != 1) continue;
+                a = __ldg(&p.edge[v].a);
+            } else {
+                q = perimeter_of(v, p.start, p.n_poly);
+                if (p.kind[q] != 1) continue;
+                const CostmapEdge e = make_edge(p, v, q);
+                a = e.a;
+                b = e.b;
+            }
+            const bool near = !(fmaxf(a.x, b.x) + reach < tx0 || fminf(a.x, b.x) - reach > tx1 ||
+                                fmaxf(a.y, b.y) + reach < ty0 || fminf(a.y, b.y) - reach > ty1);
+            if (near) atomicOr(&s_near[q], 2);
+            if (crosses(a, b, mx, my)) atomicXor(&s_near[q], 1);
+        }
+        __syncthreads();
+    }
+    // the perimeters that count here, in their order, by a block-wide scan
+    // over one thread per perimeter
     bool keep = false;
     int nv = 0;
     if (t < p.n_poly) {
         keep = true;
-        if (p.box && p.kind[t] == 0) {
-            const float tx0 = (float)((double)(blockIdx.x * 16) * p.cell);
-            const float tx1 = (float)((double)(blockIdx.x * 16 + 15) * p.cell);
-            const float ty0 = (float)((double)(blockIdx.y * 16) * p.cell);
-            const float ty1 = (float)((double)(blockIdx.y * 16 + 15) * p.cell);
-            const float4 b = p.box[t];
-            keep = !(b.z < tx0 || b.x > tx1 || b.w < ty0 || b.y > ty1);
+        if (!all) {
+            if (p.kind[t] == 0) {
+                const float4 b = p.box[t];
+                keep = !(b.z < tx0 || b.x > tx1 || b.w < ty0 || b.y > ty1);
+            } else {
+                keep = s_near[t] != 1;
+            }
         }
         nv = keep ? p.start[t + 1] - p.start[t] : 0;
     }
@@ -351,83 +512,91 @@ __global__ void __launch_bounds__(256) costmap_kernel(const __grid_constant__ Co
         s_off[k] = bv + inc - nv;
     }
     if (t == 0) s_off[n_keep] = n_vert;
-    float c = 0.f, smin = CUDART_INF_F;
+    const float px = s_x[threadIdx.x];
+    float py[kRows], c[kRows], smin[kRows], d2[kRows];
+    bool inside[kRows];
+#pragma unroll
+    for (int m = 0; m < kRows; ++m) {
+        py[m] = s_y[threadIdx.y + 8 * m];
+        c[m] = 0.f;
+        smin[m] = d2[m] = CUDART_INF_F;
+        inside[m] = false;
+    }
     int cur = -1;
-    float d2 = CUDART_INF_F;
-    bool inside = false;
     // the signed distance of the polygon just finished and its cost
-    auto finish = [&](int q) {
-        const float d = sqrtf(d2);
-        const bool neg = p.kind[q] == 0 ? inside : !inside;
-        const float s = neg ? -d : d;
-        const float v = 1.f - s * p.inv_eps;
-        if (v > 0.f) c = fmaf(p.sigma * v, v, c);
-        smin = fminf(smin, s);
+    const auto finish = [&](int q) {
+        const bool path = p.kind[q] != 0;
+#pragma unroll
+        for (int m = 0; m < kRows; ++m) {
+            const float d = sqrtf(d2[m]);
+            const float s = inside[m] != path ? -d : d;
+            const float v = 1.f - s * p.inv_eps;
+            if (v > 0.f) c[m] = fmaf(p.sigma * v, v, c[m]);
+            smin[m] = fminf(smin[m], s);
+            d2[m] = CUDART_INF_F;
+            inside[m] = false;
+        }
     };
     for (int c0 = 0; c0 < n_vert; c0 += kChunk) {
         __syncthreads();
         const int vc = c0 + t;
         if (vc < n_vert) {
-            int lo = 0, hi = n_keep;               // s_off[lo] <= vc < s_off[lo + 1]
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (s_off[mid] <= vc) lo = mid;
-                else hi = mid;
+            const int lo = perimeter_of(vc, s_off, n_keep);
+            const int v = p.start[s_id[lo]] + (vc - s_off[lo]);
+            if (p.edge) {
+                s_a[t] = __ldg(&p.edge[v].a);
+                s_b[t] = __ldg(&p.edge[v].b);
+            } else {
+                const CostmapEdge e = make_edge(p, v, s_id[lo]);
+                s_a[t] = e.a;
+                s_b[t] = e.b;
             }
-            const int q = s_id[lo];
-            const int v = p.start[q] + (vc - s_off[lo]);
-            const int nxt = v + 1 < p.start[q + 1] ? v + 1 : p.start[q];
-            s_a[t] = make_float2((float)(p.xy[2 * v] - p.x0), (float)(p.xy[2 * v + 1] - p.y0));
-            s_b[t] = make_float2((float)(p.xy[2 * nxt] - p.x0), (float)(p.xy[2 * nxt + 1] - p.y0));
-            s_poly[t] = q;
         }
         __syncthreads();
-        const int m = min(kChunk, n_vert - c0);
-        for (int e = 0; e < m; ++e) {
-            const int q = s_poly[e];
+        const int m_e = min(kChunk, n_vert - c0);
+        for (int e = 0; e < m_e; ++e) {
+            const float4 a = s_a[e], b = s_b[e];
+            const int q = __float_as_int(b.w);
             if (q != cur) {
                 if (cur >= 0) finish(cur);
                 cur = q;
-                d2 = CUDART_INF_F;
-                inside = false;
             }
-            const float2 a = s_a[e], b = s_b[e];
-            // distance to the segment a-b
-            const float ex = b.x - a.x, ey = b.y - a.y;
-            const float rx = px - a.x, ry = py - a.y;
-            const float l2 = fmaf(ex, ex, ey * ey);
-            float u = l2 > 0.f ? fmaf(rx, ex, ry * ey) / l2 : 0.f;
-            u = fminf(fmaxf(u, 0.f), 1.f);
-            const float dx = px - fmaf(u, ex, a.x), dy = py - fmaf(u, ey, a.y);
-            d2 = fminf(d2, fmaf(dx, dx, dy * dy));
-            // even-odd rule, ray towards +x
-            if ((a.y > py) != (b.y > py)) {
-                const float xc = fmaf((py - a.y) / (b.y - a.y), ex, a.x);
-                if (px < xc) inside = !inside;
+            const float rx = px - a.x;
+#pragma unroll
+            for (int m = 0; m < kRows; ++m) {
+                // distance to the segment
+                const float ry = py[m] - a.y;
+                float u = b.z > 0.f ? fmaf(rx, a.z, ry * a.w) / b.z : 0.f;
+                u = fminf(fmaxf(u, 0.f), 1.f);
+                const float dx = px - fmaf(u, a.z, a.x), dy = py[m] - fmaf(u, a.w, a.y);
+                d2[m] = fminf(d2[m], fmaf(dx, dx, dy * dy));
+                inside[m] = inside[m] != crosses(a, b, px, py[m]);
             }
         }
     }
     if (cur >= 0) finish(cur);
-    if (!live) return;
-    const size_t o = (size_t)j * p.nx + i;
-    p.cost[o] = c;
-    if (p.sdist) p.sdist[o] = smin;
+    const int i = blockIdx.x * kTile + threadIdx.x;
+    if (i >= p.nx) return;
+#pragma unroll
+    for (int m = 0; m < kRows; ++m) {
+        const int j = blockIdx.y * kTile + threadIdx.y + 8 * m;
+        if (j >= p.ny) return;
+        const size_t o = (size_t)j * p.nx + i;
+        p.cost[o] = c[m];
+        if (all) p.sdist[o] = smin[m];
+    }
 }
 
 }  // namespace
 
-cudaError_t launch_costmap(CostmapParams p, float4 *box_buf, float reach, cudaStream_t stream)
+cudaError_t launch_costmap(const CostmapParams &p, float reach, cudaStream_t stream)
 {
     if (p.n_poly < 1 || p.n_poly > kCostmapMaxPolys) return cudaErrorInvalidValue;
-    p.box = nullptr;
-    if (box_buf && !p.sdist) {
-        costmap_boxes_kernel<<<(unsigned)p.n_poly, 32, 0, stream>>>(p, box_buf, reach);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        p.box = box_buf;
-    }
-    const dim3 grid((unsigned)((p.nx + 15) / 16), (unsigned)((p.ny + 15) / 16));
-    costmap_kernel<<<grid, dim3(16, 16), 0, stream>>>(p);
+    costmap_edges_kernel<<<(unsigned)p.n_poly, 32, 0, stream>>>(p, reach);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((p.nx + kTile - 1) / kTile), (unsigned)((p.ny + kTile - 1) / kTile));
+    costmap_kernel<<<grid, dim3(32, 8), 0, stream>>>(p, reach);
     return cudaGetLastError();
 }
 

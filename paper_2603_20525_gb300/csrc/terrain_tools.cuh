@@ -24,10 +24,17 @@ cudaError_t launch_lod_smooth(const float *in, float *tmp, float *out, int nx, i
                               float inv2s2, cudaStream_t stream);
 
 constexpr int kCostmapMaxPolys = 256;
+constexpr int kCostmapEdges = 16384;     // edges kept between the costmap's kernels
+
+// One edge from (a.x, a.y) along (a.z, a.w) to (b.x, b.y): its squared length
+// b.z and its perimeter's index b.w (as bits).
+struct CostmapEdge {
+    float4 a, b;
+};
 
 struct CostmapParams {
     const double *xy;         // vertices [n_vert][2], world metres
-    int n_poly, n_vert;
+    int n_poly, n_vert, n_path;        // perimeters, vertices, path boundaries
     int start[kCostmapMaxPolys + 1];   // polygon p: vertices start[p] .. start[p+1]-1
     int kind[kCostmapMaxPolys];        // 0 obstacle, 1 path boundary
     int nx, ny;
@@ -35,16 +42,16 @@ struct CostmapParams {
     float inv_eps, sigma;
     float *cost;              // [ny][nx]
     float *sdist;             // [ny][nx] or nullptr: smallest signed distance
-    const float4 *box;        // [n_poly] reach boxes (set by launch_costmap) or nullptr
+    float4 *box;              // [n_poly] scratch: the perimeters' boxes
+    CostmapEdge *edge;        // [n_vert] scratch, or nullptr above kCostmapEdges (made on use)
 };
 
-// With box_buf (device, kCostmapMaxPolys float4) and no sdist output, a first
-// kernel writes each perimeter's bounding box grown by `reach` metres and the
-// costmap kernel skips, per 16 x 16 tile of nodes, every obstacle whose grown
-// box misses the tile: beyond `reach` (at least twice eps) its cost rate is
-// exactly zero, so the costmap keeps its bits.  Path boundaries are never
-// skipped (their cost lies outside them), nor is anything when sdist is
-// wanted (the smallest distance needs every perimeter).
-cudaError_t launch_costmap(CostmapParams p, float4 *box_buf, float reach, cudaStream_t stream);
+// A first kernel writes each perimeter's edges and bounding box (grown by
+// `reach` metres); the costmap kernel leaves out, per 32 x 32 tile of nodes, the
+// perimeters whose cost rate is exactly zero at every one of its nodes: beyond
+// `reach` (at least twice eps) outside an obstacle or inside a path boundary.
+// Nothing is left out when sdist is wanted (the smallest distance needs every
+// perimeter).  The costmap has the same bits either way.
+cudaError_t launch_costmap(const CostmapParams &p, float reach, cudaStream_t stream);
 
 }  // namespace atp

@@ -9,7 +9,10 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 import threading
+from itertools import accumulate
+from operator import itemgetter
 
 from . import build as _build
 
@@ -143,16 +146,42 @@ def load(build_if_missing: bool = True):
         return L
 
 
+# A struct's fields packed in one go (about 2 us instead of 10 for a vehicle, on
+# every call); values that the packing refuses (texts, numbers beyond FP32) go
+# through float() and ctypes one by one.
+def _packer(cls, code):
+    names = tuple(n for n, _ in cls._fields_)
+    pack, get, new = struct.Struct(f"{len(names)}{code}").pack, itemgetter(*names), cls.from_buffer_copy
+    return names, pack, get, new
+
+
+_VEH, _COST, _STATE = _packer(Vehicle, "d"), _packer(Cost, "d"), _packer(State, "f")
+_REFUSED = (struct.error, TypeError, OverflowError)
+
+
 def vehicle(d: dict) -> Vehicle:
-    return Vehicle(**{k: float(d[k]) for k, _ in Vehicle._fields_})
+    names, pack, get, new = _VEH
+    try:
+        return new(pack(*get(d)))
+    except _REFUSED:
+        return Vehicle(**{k: float(d[k]) for k in names})
 
 
 def cost(d: dict) -> Cost:
-    return Cost(**{k: float(d[k]) for k, _ in Cost._fields_})
+    names, pack, get, new = _COST
+    try:
+        return new(pack(*get(d)))
+    except _REFUSED:
+        return Cost(**{k: float(d[k]) for k in names})
 
 
 def state(x) -> State:
-    return State(*[float(v) for v in x])
+    _, pack, _, new = _STATE
+    x = tuple(x)
+    try:
+        return new(pack(*x))
+    except _REFUSED:
+        return State(*[float(v) for v in x])
 
 
 class AtpError(RuntimeError):
@@ -160,13 +189,16 @@ class AtpError(RuntimeError):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class Terrain:
@@ -306,11 +338,14 @@ class Context:
         kind) with kind 0 obstacle, 1 path boundary."""
         import numpy as np
         import torch
-        xy = np.concatenate([np.asarray(p, np.float64).reshape(-1, 2) for p, _ in polys])
-        start = (C.c_int * (len(polys) + 1))(0, *np.cumsum([len(np.asarray(p).reshape(-1, 2))
-                                                            for p, _ in polys]).tolist())
+        verts = [np.asarray(p, np.float64).reshape(-1, 2) for p, _ in polys]
+        xy = torch.from_numpy(np.concatenate(verts))
+        start = (C.c_int * (len(polys) + 1))(0, *accumulate(len(v) for v in verts))
         kind = (C.c_int * len(polys))(*[int(k) for _, k in polys])
-        xy_d = torch.as_tensor(xy, device=device)
+        # from pinned memory on the call's own stream, so that the copy waits
+        # for nothing
+        with torch.cuda.stream(stream):
+            xy_d = xy.pin_memory().to(device, non_blocking=True)
         cm = torch.empty((ny, nx), dtype=torch.float32, device=device)
         sd = torch.empty((ny, nx), dtype=torch.float32, device=device) if want_sdist else None
         rc = self.lib.atp_costmap(self.h, _ptr(xy_d), start, kind, len(polys), int(nx), int(ny),

@@ -90,3 +90,40 @@ def test_degenerate_starts(ctx):
     one = plan(ctx, w, x0, 1)
     for lanes in (2, 4):
         same(plan(ctx, w, x0, lanes), one)
+
+
+@pytest.mark.parametrize("acc64,n_sub,costmap", [(0, 4, False), (1, 3, True)])
+def test_planar_plan(ctx, acc64, n_sub, costmap):
+    """The planar plan's two-warp form (up to 48640 candidates) against one
+    thread per candidate (more of them, the same ones repeated)."""
+    from paper_2603_20525_gb300 import atp
+    w = gen.workload_est(0, N=70, H=25)
+    s = np.repeat(w.x0[None, :], 70, 0)
+    s[:, 6] = (1.0 + 12.0 * gen.uniform(5, 6, 70)).astype(np.float32)
+    for i, (q, v) in enumerate([(0, -5.0), (1, 1e9), (2, 3.0), (2, -1e7), (5, 2e5), (3, 1e20), (4, 1e6)]):
+        s[3 + i, q] = v
+    for q in range(7):
+        s[20 + q, q], s[40 + q, q] = np.nan, np.inf
+    cost = gen.cost_default(14.0, 25.6)
+    cm = dev(gen.uniform(4, 6, 256 * 256).reshape(256, 256).astype(np.float32)) if costmap else None
+    ter = ctx.terrain_prepare(dev(w.terrain.heights), w.terrain.cell, costmap=cm)
+    ctx.set_option(atp.OPT_COST_FP64, acc64)
+    try:
+        r = {}
+        for N in (1, 33, 70, 48640, 48641):
+            i = np.arange(N) % 70
+            o = ctx.plan_est(w.vehicle, cost, ter, dev(s[i].T.copy()), dev(w.ctrl[:, i]), w.dt, n_sub, want_xf=True)
+            torch.cuda.synchronize()
+            r[N] = {k: v.cpu().numpy() for k, v in o.items()}
+    finally:
+        ctx.set_option(atp.OPT_COST_FP64, 0)
+    one = r[48641]
+    assert 0 < np.sum(one["flags"][:70] & 2) // 2 < 70
+    for N in (1, 33, 70, 48640):
+        for k in ("cost", "margin", "flags", "xf"):
+            assert np.array_equal(r[N][k], one[k][..., :N], equal_nan=k != "flags"), (N, k)
+    for k in ("best_ctrl", "best_margin", "out"):
+        a, b = r[70][k], r[48640][k]
+        if k == "out":
+            a, b = np.delete(a, 1), np.delete(b, 1)          # not the feasible count
+        assert np.array_equal(a, b), k

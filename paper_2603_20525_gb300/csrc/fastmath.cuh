@@ -98,8 +98,6 @@ __device__ __forceinline__ void sincos_g(float x, float &s, float &c)
     c = __uint_as_float(__float_as_uint(odd ? sr : cr) ^ (((q + 1u) & 2u) << 30));
     if (SLOW && fabsf(x) >= kSincosMax) sincosf(x, &s, &c);
 }
-__device__ __forceinline__ void sincos_b(float x, float &s, float &c) { sincos_g<true>(x, s, c); }
-
 // atan(r) for r in [0, 1] as r P(r^2), P of degree 8 fitted for minimum
 // maximum relative error (fit_atan.py): 1.1e-7 including FP32 evaluation.
 __device__ __forceinline__ float atan01(float r)

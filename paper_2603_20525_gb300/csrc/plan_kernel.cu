@@ -29,9 +29,10 @@
 
 namespace atp {
 
-// One thread per candidate.  The heading's sincos takes the reduction without
-// a branch (headings spread over the circle, so a warp ran both paths); roll,
-// pitch and steering stay mostly below pi/4 and keep it.
+// One thread per candidate.  The four sincos take the reduction without a
+// branch, one test covering their slow form: headings spread over the circle
+// and tipped candidates' roll and pitch grow, so that warps ran both paths of
+// each (paper configuration 4.84 -> 4.41 ms, 50000 x 100 x 4 steps 664 -> 639 us).
 template <bool PER_X0, int TEX, int ACC>
 __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J, float &margin, bool &feasible)
 {
@@ -88,9 +89,17 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J
                     continue;
                 }
                 float sps, cps, sth, cth, sph, cph;
-                sincos_b(psi, sps, cps);
-                sincos_r(th, sth, cth);
-                sincos_r(ph, sph, cph);
+                float sd, cd;
+                sincos_g<false>(d, sd, cd);
+                sincos_g<false>(psi, sps, cps);
+                sincos_g<false>(th, sth, cth);
+                sincos_g<false>(ph, sph, cph);
+                if (fmaxf(fmaxf(fabsf(psi), fabsf(d)), fmaxf(fabsf(th), fabsf(ph))) >= kSincosMax) {
+                    sincos_g<true>(psi, sps, cps);
+                    sincos_g<true>(th, sth, cth);
+                    sincos_g<true>(ph, sph, cph);
+                    sincos_g<true>(d, sd, cd);
+                }
                 const float U = esm(V, ph, sph, cph, cth);
                 margin = fminf(margin, U);
                 sm = fminf(sm, U);
@@ -124,8 +133,6 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J
                 B.wx = wx; B.wy = wy; B.wz = wz;
                 // gravity in B: R^T (0, 0, -g)
                 const float gBx = -V.g * R[6], gBy = -V.g * R[7], gBz = -V.g * R[8];
-                float sd, cd;
-                sincos_r(d, sd, cd);
                 // summed forces and moments (Sec. IV-A); the rear
                 // longitudinal constraint force enters My only
                 const WheelOut fl = wheel<TEX>(V, T, B, V.Lf, V.he, V.kf, V.bf, V.Fsf, d, off);
@@ -227,10 +234,10 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J
 
 }
 
-// Five CTAs per SM leave ptxas 168 registers and no spills: 4.75 ms on the
-// paper configuration against 4.84 ms at six and 4.87 ms at seven (128
-// registers, 32 B of spills; the lookups' map edges keep more values live
-// than the integer clamps they replaced).
+// Five CTAs per SM leave ptxas 168 registers and no spills: 2 % faster on the
+// paper configuration than at six or seven (128 registers, 32 B of spills; the
+// lookups' map edges keep more values live than the integer clamps they
+// replaced) and 10 % than at four.
 template <bool PER_X0, bool REDUCE, int TEX, int ACC>
 __global__ void __launch_bounds__(kPlanBlock, 5)
 plan_kernel(const __grid_constant__ PlanParams p)

@@ -336,7 +336,7 @@ int choose_layout(const atp_plan_request *q, const int *ns, int n)
     // cycles per Euler step with the GPU nearly idle, and SM cycles per
     // candidate and Euler step with it full, from a sweep on a GB300
     constexpr int kL[4] = {atp::kLayoutOne, atp::kLayoutDuo1, atp::kLayoutDuo2, atp::kLayoutDuo4};
-    constexpr double kLatency[4] = {1744., 1273., 1000., 818.}, kBusy[4] = {9.0, 10.3, 12.9, 19.5};
+    constexpr double kLatency[4] = {1744., 1200., 1000., 810.}, kBusy[4] = {9.0, 10.3, 12.9, 26.};
     constexpr double kSms = 152., kWave = 6 * kSms;
     double best = INFINITY;
     int layout = atp::kLayoutOne;

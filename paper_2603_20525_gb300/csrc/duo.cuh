@@ -69,9 +69,9 @@ template <int LANES>
 struct Duo {
     static constexpr int kW = 4 / LANES;            // wheels per lane
     static constexpr int kC = 32 / LANES;           // candidates per pair of warps
-    float4 tau[2][kW][32];                          // tx, ty, tz, 1 / tz per wheel
-    float2 chi[2][kW][32];                          // extension, costmap
+    float4 ground[2][kW][32];                       // WheelGround per wheel
     float4 att[2][kC];                              // sin and cos of theta, then of phi
+    float2 yaw[2][kC];                              // sin and cos of psi
     float4 body[2][kC];                             // delta, cos(delta), phi; done (0 or 1)
     float4 va[2][kC];                               // vx, vy, vz, wx
     float2 vb[2][kC];                               // wy, wz
@@ -214,22 +214,14 @@ __device__ __forceinline__ void duo_geometry(const PlanParams &p, const Tr &tr, 
             cph = sel(q1, oc2, c2);
             cdl = sel(q1, c2, oc2);
         }
-        // 3-2-1 rotation, body -> world (Sec. IV-A)
-        R[0] = cps * cth;
-        R[1] = fmaf(cps * sph, sth, -cph * sps);
-        R[2] = fmaf(cph * cps, sth, sph * sps);
-        R[3] = cth * sps;
-        R[4] = fmaf(sph * sps, sth, cph * cps);
-        R[5] = fmaf(cph * sps, sth, -cps * sph);
-        R[6] = -sth;
-        R[7] = cth * sph;
-        R[8] = cph * cth;
+        rotation(sps, cps, sth, cth, sph, cph, R);
         // goal test before the step (Sec. IV-C, reading Q4)
         const float gdx = (x - Cc.gx_hi) + (xl - Cc.gx_lo);
         const float gdy = (y - Cc.gy_hi) + (yl - Cc.gy_lo);
         done = done || fmaf(gdx, gdx, gdy * gdy) <= Cc.goal_r2;
         if (q == 0) {
             sh.att[par][c] = make_float4(sth, cth, sph, cph);
+            sh.yaw[par][c] = make_float2(sps, cps);
             sh.body[par][c] = make_float4(d, cdl, ph, done ? 1.f : 0.f);
         }
         const Cell cx = cell_of<!Tr::on>(x, xl, T.inv_cell, T.nx), cy = cell_of<!Tr::on>(y, yl, T.inv_cell, T.ny);
@@ -237,10 +229,9 @@ __device__ __forceinline__ void duo_geometry(const PlanParams &p, const Tr &tr, 
         offs = off_com(cx, cy);
     #pragma unroll
         for (int w = 0; w < Duo<LANES>::kW; ++w) {
-            const WheelGeo g = wheel_geo<TEX>(V, T, R, cx, cy, base, z, zl, w < 2 ? lw.rx : -V.Lr,
-                                              LANES == 4 ? lw.ry : (w & 1) ? -V.he : V.he, offs);
-            sh.tau[par][w][lane] = make_float4(g.tx, g.ty, g.tz, g.itz);
-            sh.chi[par][w][lane] = make_float2(g.chi, g.cost);
+            const WheelGround g = wheel_ground<TEX>(V, T, R, cx, cy, base, z, zl, w < 2 ? lw.rx : -V.Lr,
+                                                    LANES == 4 ? lw.ry : (w & 1) ? -V.he : V.he, offs);
+            sh.ground[par][w][lane] = make_float4(g.fx, g.fy, g.Q, g.cost);
         }
     };
 
@@ -420,14 +411,18 @@ __device__ __forceinline__ void duo_forces(const PlanParams &p, const Tr &tr, Du
                 // summed forces and moments (Sec. IV-A); the rear
                 // longitudinal constraint force enters My only
                 float FyB, FzB, Mx, My, Mz, csum = 0.f;
-                const float4 t0 = sh.tau[par][0][lane];
-                const float2 x0 = sh.chi[par][0][lane];
-                const WheelGeo g0 = {t0.x, t0.y, t0.z, t0.w, x0.x, x0.y};
+                // the rotation again, which the forces warp has time for
+                const float2 yaw = sh.yaw[par][c];
+                float R[9];
+                rotation(yaw.x, yaw.y, sth, cth, sph, cph, R);
+                const auto geo = [&](int w) {
+                    const float4 t = sh.ground[par][w][lane];
+                    return wheel_geo(R, WheelGround{t.x, t.y, t.z, t.w});
+                };
+                const WheelGeo g0 = geo(0);
                 if constexpr (LANES == 1) {
                     const auto wh = [&](int i, float rx, float ry, float k, float b, float Fs, float dw) {
-                        const float4 t = sh.tau[par][i][lane];
-                        const float2 x = sh.chi[par][i][lane];
-                        const WheelGeo g = {t.x, t.y, t.z, t.w, x.x, x.y};
+                        const WheelGeo g = i == 0 ? g0 : geo(i);
                         return wheel_dyn<false, Tr::on>(V, g, vx, vy, vz, wx, wy, wz, rx, ry, k, b, Fs, dw);
                     };
                     const WheelOut fl = wh(0, V.Lf, V.he, V.kf, V.bf, V.Fsf, di), fr = wh(1, V.Lf, -V.he, V.kf, V.bf, V.Fsf, di);
@@ -449,9 +444,7 @@ __device__ __forceinline__ void duo_forces(const PlanParams &p, const Tr &tr, Du
                     }
                     csum = (fl.cost + fr.cost) + (rl.cost + rr.cost);
                 } else if constexpr (LANES == 2) {
-                    const float4 t1 = sh.tau[par][1][lane];
-                    const float2 x1 = sh.chi[par][1][lane];
-                    const WheelGeo g1 = {t1.x, t1.y, t1.z, t1.w, x1.x, x1.y};
+                    const WheelGeo g1 = geo(1);
                     const WheelOut l = wheel_dyn<true, Tr::on>(V, g0, vx, vy, vz, wx, wy, wz, lw.rx, V.he, lw.k, lw.b, lw.Fs, di);
                     const WheelOut r = wheel_dyn<true, Tr::on>(V, g1, vx, vy, vz, wx, wy, wz, lw.rx, -V.he, lw.k, lw.b, lw.Fs, di);
                     FzB = pair_sum(l.Fz + r.Fz);

@@ -114,15 +114,7 @@ __device__ __forceinline__ void rollout_one(const PlanParams &p, int j, float &J
                 // 3-2-1 rotation, body -> world (Sec. IV-A)
                 Body B;
                 float *R = B.R;
-                R[0] = cps * cth;
-                R[1] = fmaf(cps * sph, sth, -cph * sps);
-                R[2] = fmaf(cph * cps, sth, sph * sps);
-                R[4] = fmaf(sph * sps, sth, cph * cps);
-                R[5] = fmaf(cph * sps, sth, -cps * sph);
-                R[3] = cth * sps;
-                R[6] = -sth;
-                R[7] = cth * sph;
-                R[8] = cph * cth;
+                rotation(sps, cps, sth, cth, sph, cph, R);
                 B.cx = cell_of(x, xl, T.inv_cell, T.nx);
                 B.cy = cell_of(y, yl, T.inv_cell, T.ny);
                 B.base = texel_base(B.cx, B.cy, T.nx);

@@ -271,14 +271,19 @@ struct WheelGeo {
     float tx, ty, tz, itz, chi, cost;
 };
 
-// One wheel's geometry (Sec. IV-A): contact point P = p + R rho, the terrain
-// below it, the slope-normal tau ~ (-f_x, -f_y, 1) (reading Q1) resolved in
-// B and the extension chi along it.  cx, cy is the CoM's cell and z_hi + z_lo
-// its height.
+// What the lookup at one wheel gives: the interpolated slopes, the CoM height
+// above the terrain there P_z - f (with the compensated CoM height), the
+// costmap.
+struct WheelGround {
+    float fx, fy, Q, cost;
+};
+
+// One wheel's ground (Sec. IV-A): contact point P = p + R rho and the terrain
+// below it.  cx, cy is the CoM's cell and z_hi + z_lo its height.
 template <int TEX>
-__device__ __forceinline__ WheelGeo wheel_geo(const Veh &V, const Terrain &T, const float R[9], const Cell &cx,
-                                              const Cell &cy, unsigned base, float z_hi, float z_lo, float rx,
-                                              float ry, bool &off)
+__device__ __forceinline__ WheelGround wheel_ground(const Veh &V, const Terrain &T, const float R[9], const Cell &cx,
+                                                    const Cell &cy, unsigned base, float z_hi, float z_lo, float rx,
+                                                    float ry, bool &off)
 {
     // offset of the contact point from the CoM in W: R (rx, ry, -(h+R))
     const float2 oxy = fma2(splat2(rx), make_float2(R[0], R[3]),
@@ -290,18 +295,38 @@ __device__ __forceinline__ WheelGeo wheel_geo(const Veh &V, const Terrain &T, co
     float a, bb;
     const float tx = axis(cx, u.x, a, off), ty = axis(cy, u.y, bb, off);
     const float4 t = bilerp<TEX>(T, cx, cy, base, tx, ty, a, bb);
+    return {t.y, t.z, (z_hi - t.x) + (oz + z_lo), t.w};
+}
+
+// The slope-normal tau ~ (-f_x, -f_y, 1) (reading Q1) resolved in B and the
+// extension chi along it.
+__device__ __forceinline__ WheelGeo wheel_geo(const float R[9], const WheelGround &t)
+{
     // tau in B = R^T (-f_x, -f_y, 1)
-    const float2 txy = fma2(make_float2(-R[3], -R[4]), splat2(t.z),
-                            fma2(make_float2(-R[0], -R[1]), splat2(t.y), make_float2(R[6], R[7])));
+    const float2 txy = fma2(make_float2(-R[3], -R[4]), splat2(t.fy),
+                            fma2(make_float2(-R[0], -R[1]), splat2(t.fx), make_float2(R[6], R[7])));
     WheelGeo g;
     g.tx = txy.x;
     g.ty = txy.y;
-    g.tz = fmaf(-R[5], t.z, fmaf(-R[2], t.y, R[8]));
+    g.tz = fmaf(-R[5], t.fy, fmaf(-R[2], t.fx, R[8]));
     g.itz = rcp(g.tz);
-    // P_z - f with the compensated CoM height
-    g.chi = ((z_hi - t.x) + (oz + z_lo)) * g.itz;
-    g.cost = t.w;
+    g.chi = t.Q * g.itz;
+    g.cost = t.cost;
     return g;
+}
+
+// 3-2-1 rotation, body -> world (Sec. IV-A)
+__device__ __forceinline__ void rotation(float sps, float cps, float sth, float cth, float sph, float cph, float R[9])
+{
+    R[0] = cps * cth;
+    R[1] = fmaf(cps * sph, sth, -cph * sps);
+    R[2] = fmaf(cph * cps, sth, sph * sps);
+    R[3] = cth * sps;
+    R[4] = fmaf(sph * sps, sth, cph * cps);
+    R[5] = fmaf(cph * sps, sth, -cps * sph);
+    R[6] = -sth;
+    R[7] = cth * sph;
+    R[8] = cph * cth;
 }
 
 // What one wheel contributes to the force and moment sums.
@@ -360,7 +385,8 @@ template <int TEX>
 __device__ __forceinline__ WheelOut wheel(const Veh &V, const Terrain &T, const Body &B, float rx, float ry,
                                           float k, float b, float Fs, float di, bool &off)
 {
-    const WheelGeo g = wheel_geo<TEX>(V, T, B.R, B.cx, B.cy, B.base, B.z_hi, B.z_lo, rx, ry, off);
+    const WheelGeo g =
+        wheel_geo(B.R, wheel_ground<TEX>(V, T, B.R, B.cx, B.cy, B.base, B.z_hi, B.z_lo, rx, ry, off));
     return wheel_dyn(V, g, B.vx, B.vy, B.vz, B.wx, B.wy, B.wz, rx, ry, k, b, Fs, di);
 }
 

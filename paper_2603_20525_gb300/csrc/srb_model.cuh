@@ -224,17 +224,34 @@ __device__ __forceinline__ float block_plane(float4 P, int i, int j)
     return __fadd_rn(__fadd_rn(P.x, __fmul_rn(P.y, (float)(i & 7))), __fmul_rn(P.z, (float)(j & 7)));
 }
 
-// one BF16 texel decoded: height = block plane + residual
-__device__ __forceinline__ float4 texel16(const Terrain &T, int i, int j)
+// one BF16 texel decoded from its block's plane, at (x, y) within the block:
+// height = block plane + residual
+__device__ __forceinline__ float4 texel16(const Terrain &T, uint2 u, float4 P, float x, float y)
 {
-    const uint2 u = __ldg(T.tex16 + (size_t)j * T.nx + i);
-    const float4 P = __ldg(T.plane16 + (size_t)(j >> 3) * T.nbx + (i >> 3));
     float4 t;
-    t.x = __fadd_rn(block_plane(P, i, j), __uint_as_float(u.x << 16));
+    t.x = __fadd_rn(__fadd_rn(__fadd_rn(P.x, __fmul_rn(P.y, x)), __fmul_rn(P.z, y)), __uint_as_float(u.x << 16));
     t.y = __fadd_rn(__fmul_rn(P.y, T.inv_cell), __uint_as_float(u.x & 0xffff0000u));
     t.z = __fadd_rn(__fmul_rn(P.z, T.inv_cell), __uint_as_float(u.y << 16));
     t.w = __uint_as_float(u.y & 0xffff0000u);
     return t;
+}
+
+// v mod 8 as a float, by its bits
+__device__ __forceinline__ float mod8(int v) { return __uint_as_float(0x4b000000u | (unsigned)(v & 7)) - 8388608.f; }
+
+// Bilinear lookup on BF16 texels.  The four corners mostly share one block, but
+// loading the other planes only in the lanes that straddle an edge was slower
+// (branches on the lookup's chain).
+__device__ __forceinline__ float4 bilerp16(const Terrain &T, int i, int j, float a, float b, bool cm)
+{
+    const uint2 *r0 = T.tex16 + (size_t)j * T.nx + i, *r1 = r0 + T.nx;
+    const uint2 u00 = __ldg(r0), u10 = __ldg(r0 + 1), u01 = __ldg(r1), u11 = __ldg(r1 + 1);
+    const float4 *P = T.plane16 + (size_t)(j >> 3) * T.nbx + (i >> 3);
+    const int ex = ((i & 7) + 1) >> 3, ey = ((j & 7) + 1) >> 3 ? T.nbx : 0;
+    const float4 P00 = __ldg(P), P10 = __ldg(P + ex), P01 = __ldg(P + ey), P11 = __ldg(P + ex + ey);
+    const float x0 = mod8(i), x1 = mod8(i + 1), y0 = mod8(j), y1 = mod8(j + 1);
+    return lerp4(texel16(T, u00, P00, x0, y0), texel16(T, u10, P10, x1, y0), texel16(T, u01, P01, x0, y1),
+                 texel16(T, u11, P11, x1, y1), a, b, cm);
 }
 
 // The lookup at cell (tx, ty) (magic form) with weights (a, b), seen from the
@@ -258,9 +275,7 @@ __device__ __forceinline__ float4 bilerp(const Terrain &T, const Cell &cx, const
         const int s = in ? T.ww : T.nx;
         return lerp4(r0[0], r0[1], r0[s], r0[s + 1], a, b, cm);
     } else {
-        const int i = cell_index(cx, tx), j = cell_index(cy, ty);
-        return lerp4(texel16(T, i, j), texel16(T, i + 1, j), texel16(T, i, j + 1),
-                     texel16(T, i + 1, j + 1), a, b, cm);
+        return bilerp16(T, cell_index(cx, tx), cell_index(cy, ty), a, b, cm);
     }
 }
 

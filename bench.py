@@ -67,6 +67,7 @@ def fp32_peak_tflops(sms, mhz):
 # what the plan kernel is compiled from: its translation unit, the headers it
 # includes and the module that holds the compile flags
 PLAN_KERNEL_SOURCES = ("paper_2603_20525_gb300/csrc/plan_kernel.cu", "paper_2603_20525_gb300/csrc/plan_kernel.cuh",
+                       "paper_2603_20525_gb300/csrc/duo.cuh", "paper_2603_20525_gb300/csrc/adjoint.cuh",
                        "paper_2603_20525_gb300/csrc/plan_tail.cuh", "paper_2603_20525_gb300/csrc/srb_model.cuh",
                        "paper_2603_20525_gb300/csrc/fastmath.cuh", "include/atp.h",
                        "paper_2603_20525_gb300/build.py")
@@ -436,8 +437,8 @@ def run_variants(ctx, dev, stream, flush, steps=10):
     ms = _time(lambda: ctx.costmap(polys, t.nx, t.ny, t.cell, t.x0, t.y0), steps, 3, stream, flush)
     out["costmap"] = {"workload": f"2048^2 nodes, {len(polys)} perimeters, {nv} edges", "ms": ms,
                       "nodes_per_s": 2048 * 2048 / (ms / 1e3),
-                      "note": "each 16 x 16 tile skips the obstacles beyond 2 eps of it (exactly zero "
-                              "rate there); the path boundary is evaluated at every node"}
+                      "note": "each 32 x 32 tile leaves out the perimeters whose rate is exactly zero "
+                              "in it (beyond 2 eps outside an obstacle or inside the boundary)"}
     # the adjoint's configuration: 64 candidates of the plain plan at H = 100, dt = 0.02 s
     wa = gen.workload_plain(0, N=64, H=100, dt=0.02)
     tera = ctx.terrain_prepare(torch.as_tensor(wa.terrain.heights).to(dev), wa.terrain.cell)
@@ -660,7 +661,7 @@ def main():
                            "p99": float(np.percentile(per_step, 99))},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": recorded_traffic(args.workload),
-                         "kernel": "plan_kernel (fused rollout + argmin)",
+                         "kernel": "plan_duo_kernel (fused rollout + argmin)",
                          "note": f"{flops} algorithmic FP32 flops per Euler step (counted by the "
                                  f"oracle's counting scalar) x {substeps} Euler steps per launch; "
                                  f"peak = {sms} SMs (device query) x {FP32_LANES_PER_SM} FP32 lanes x 2 "

@@ -343,9 +343,16 @@ class Context:
         start = (C.c_int * (len(polys) + 1))(0, *accumulate(len(v) for v in verts))
         kind = (C.c_int * len(polys))(*[int(k) for _, k in polys])
         # from pinned memory on the call's own stream, so that the copy waits
-        # for nothing
+        # for nothing.  A graph would hold the address of that memory after it
+        # is given back: a captured copy is refused, and where only the
+        # launches are captured the copy is made at once.
+        capturing = torch.cuda.is_current_stream_capturing
+        if capturing():
+            raise RuntimeError("costmap copies its vertices from the host, which a stream capture cannot hold")
         with torch.cuda.stream(stream):
-            xy_d = xy.pin_memory().to(device, non_blocking=True)
+            xy_d = None if capturing() else xy.pin_memory().to(device, non_blocking=True)
+        if xy_d is None:
+            xy_d = xy.to(device)
         cm = torch.empty((ny, nx), dtype=torch.float32, device=device)
         sd = torch.empty((ny, nx), dtype=torch.float32, device=device) if want_sdist else None
         rc = self.lib.atp_costmap(self.h, _ptr(xy_d), start, kind, len(polys), int(nx), int(ny),

@@ -85,3 +85,23 @@ def test_texels_of_odd_maps(ctx, ny, nx):
     gy[1:-1] = (f[2:] - f[:-2]) * np.float32(2.0)
     gy[0], gy[-1] = (f[1] - f[0]) * np.float32(4.0), (f[-1] - f[-2]) * np.float32(4.0)
     assert np.array_equal(t, np.stack([f, gx, gy, cm], -1))
+
+
+def test_costmap_refuses_a_capture(ctx):
+    """The vertices' copy reads host memory that does not outlive the call, so
+    a graph that held it would read whatever lies there at its replay: refused
+    before anything is enqueued, with the context and the capture intact."""
+    box = np.array([[1.0, 1.0], [2.0, 1.0], [2.0, 2.0], [1.0, 2.0]])
+    want = ctx.costmap([(box, 0)], 40, 40, 0.1)
+    one = torch.zeros(1, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        one += 1
+        with pytest.raises(RuntimeError):
+            ctx.costmap([(box, 0)], 40, 40, 0.1)
+    g.replay()
+    again = ctx.costmap([(box, 0)], 40, 40, 0.1)
+    torch.cuda.synchronize()
+    assert one.item() == 1
+    assert torch.equal(again, want) and (want > 0).any()

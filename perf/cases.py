@@ -433,10 +433,7 @@ class _Map64:
 
     def at(self, x, y):
         u, w = (x / self.cell).clamp(0, self.nx - 1), (y / self.cell).clamp(0, self.ny - 1)
-        # a rollout that has diverged looks up at NaN: the value stays NaN, the
-        # index has to lie on the map
-        i = torch.nan_to_num(u.detach()).floor().clamp(max=self.nx - 2)
-        j = torch.nan_to_num(w.detach()).floor().clamp(max=self.ny - 2)
+        i, j = u.detach().floor().clamp(max=self.nx - 2), w.detach().floor().clamp(max=self.ny - 2)
         a, b = (u - i)[..., None], (w - j)[..., None]
         o = (j * self.nx + i).long()
         lo = self.t[o] * (1 - a) + self.t[o + 1] * a

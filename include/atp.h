@@ -409,10 +409,13 @@ int atp_lod_smooth(atp_ctx *ctx, const float *heights_dev, int nx, int ny, doubl
  *   kind        int [n_poly], host: 0 obstacle, 1 path boundary
  *   cost_dev    float [ny][nx], device
  *   sdist_dev   float [ny][nx] or NULL: the smallest signed distance
- * 1 <= n_poly <= 256.  Without sdist_dev, each 16 x 16 tile of nodes skips the
- * obstacles whose bounding box lies more than 2 eps away from it (their rate
- * there is exactly zero), which gives the same costmap bits as evaluating
- * every perimeter; with sdist_dev every perimeter is evaluated at every node. */
+ * 1 <= n_poly <= 256.  Without sdist_dev, each 32 x 32 tile of nodes leaves
+ * out the perimeters whose rate is exactly zero in all of it (more than 2 eps
+ * outside an obstacle or inside a path boundary), which gives the same costmap
+ * bits as evaluating every perimeter; a perimeter with a vertex that is not
+ * finite, or so far off that FP32 rounding there is not small against eps, is
+ * left out nowhere.  With sdist_dev every perimeter is evaluated at every
+ * node. */
 int atp_costmap(atp_ctx *ctx, const double *xy_dev, const int *start, const int *kind, int n_poly,
                 int nx, int ny, double cell, double x0, double y0, double eps, double sigma,
                 float *cost_dev, float *sdist_dev, void *stream);

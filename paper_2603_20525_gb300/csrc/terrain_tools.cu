@@ -377,15 +377,27 @@ __device__ __forceinline__ CostmapEdge make_edge(const CostmapParams &p, int v, 
     return e;
 }
 
+// Whether nothing can be said of where an edge costs anything: a vertex at
+// infinity, a NaN, or coordinates so large that the rounding of the distance
+// and of the inside test (a few parts in 2^24 of them) is no longer small
+// against `reach`.  Its perimeter is never left out of a tile.  Edges on the
+// map pass: `reach` is at least 1e-5 of its side.
+__device__ __forceinline__ bool unbounded(float4 a, float4 b, float reach)
+{
+    return !((fabsf(a.x) + fabsf(a.y)) + (fabsf(b.x) + fabsf(b.y)) < 524288.f * reach);
+}
+
 // One warp per perimeter: its edges, where they are kept, and its bounding box
-// grown by `reach`.
+// grown by `reach` (the whole plane where an edge is unbounded).
 __global__ void __launch_bounds__(32) costmap_edges_kernel(const __grid_constant__ CostmapParams p, float reach)
 {
     const int q = blockIdx.x, v0 = p.start[q], v1 = p.start[q + 1];
     float x0 = CUDART_INF_F, y0 = CUDART_INF_F, x1 = -CUDART_INF_F, y1 = -CUDART_INF_F;
+    bool whole = false;
     for (int v = v0 + (int)threadIdx.x; v < v1; v += 32) {
         const CostmapEdge e = make_edge(p, v, q);
         if (p.edge) p.edge[v] = e;
+        whole = whole || unbounded(e.a, e.b, reach);
         x0 = fminf(x0, e.a.x);
         y0 = fminf(y0, e.a.y);
         x1 = fmaxf(x1, e.a.x);
@@ -398,7 +410,10 @@ __global__ void __launch_bounds__(32) costmap_edges_kernel(const __grid_constant
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
         y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
     }
-    if (threadIdx.x == 0) p.box[q] = make_float4(x0 - reach, y0 - reach, x1 + reach, y1 + reach);
+    whole = __any_sync(0xffffffffu, whole);
+    if (threadIdx.x == 0)
+        p.box[q] = whole ? make_float4(-CUDART_INF_F, -CUDART_INF_F, CUDART_INF_F, CUDART_INF_F)
+                         : make_float4(x0 - reach, y0 - reach, x1 + reach, y1 + reach);
 }
 
 // off[k] <= v < off[k + 1]
@@ -460,7 +475,8 @@ __global__ void __launch_bounds__(256) costmap_kernel(const __grid_constant__ Co
                 a = e.a;
                 b = e.b;
             }
-            const bool near = !(fmaxf(a.x, b.x) + reach < tx0 || fminf(a.x, b.x) - reach > tx1 ||
+            const bool near = unbounded(a, b, reach) ||
+                              !(fmaxf(a.x, b.x) + reach < tx0 || fminf(a.x, b.x) - reach > tx1 ||
                                 fmaxf(a.y, b.y) + reach < ty0 || fminf(a.y, b.y) - reach > ty1);
             if (near) atomicOr(&s_near[q], 2);
             if (crosses(a, b, mx, my)) atomicXor(&s_near[q], 1);

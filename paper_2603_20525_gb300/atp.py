@@ -219,11 +219,13 @@ class Context:
         if rc != ATP_OK:
             raise AtpError(f"atp_create failed: {ERRORS.get(rc, rc)}")
         self.device = device
+        self._captured = []          # what graphs of this context's calls read, until close()
 
     def close(self):
         if self.h:
             self.lib.atp_destroy(self.h)
             self.h = C.c_void_p()
+            self._captured.clear()
 
     def __del__(self):
         try:
@@ -335,7 +337,9 @@ class Context:
                 device="cuda", stream=None):
         """Distance-constraint costmap float32 CUDA [ny, nx] (and the smallest
         signed distance) of perimeters given as a list of (vertices [n, 2],
-        kind) with kind 0 obstacle, 1 path boundary."""
+        kind) with kind 0 obstacle, 1 path boundary.  Where `stream` is being
+        captured (and is not the current stream), the graph's replays read
+        vertices that the context keeps until close()."""
         import numpy as np
         import torch
         verts = [np.asarray(p, np.float64).reshape(-1, 2) for p, _ in polys]
@@ -344,22 +348,26 @@ class Context:
         kind = (C.c_int * len(polys))(*[int(k) for _, k in polys])
         # from pinned memory on the call's own stream, so that the copy waits
         # for nothing.  A graph would hold the address of that memory after it
-        # is given back: a captured copy is refused, and where only the
-        # launches are captured the copy is made at once.
+        # is given back: a captured copy is refused.  Where only the launches
+        # are captured (the call's stream, not the current one), the copy is
+        # made at once, and the context keeps the vertices for the replays.
         capturing = torch.cuda.is_current_stream_capturing
         if capturing():
             raise RuntimeError("costmap copies its vertices from the host, which a stream capture cannot hold")
         with torch.cuda.stream(stream):
-            xy_d = None if capturing() else xy.pin_memory().to(device, non_blocking=True)
-        if xy_d is None:
+            captured = capturing()
+            if not captured:
+                xy_d = xy.pin_memory().to(device, non_blocking=True)
+        if captured:
             xy_d = xy.to(device)
+            self._captured.append(xy_d)
         cm = torch.empty((ny, nx), dtype=torch.float32, device=device)
         sd = torch.empty((ny, nx), dtype=torch.float32, device=device) if want_sdist else None
         rc = self.lib.atp_costmap(self.h, _ptr(xy_d), start, kind, len(polys), int(nx), int(ny),
                                   float(cell), float(x0), float(y0), float(eps), float(sigma),
                                   _ptr(cm), _ptr(sd), _stream(stream))
         self._check(rc, "atp_costmap")
-        if stream is not None:
+        if stream is not None and not captured:
             xy_d.record_stream(stream)
         return (cm, sd) if want_sdist else cm
 

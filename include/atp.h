@@ -289,12 +289,16 @@ int atp_plan_batch(atp_ctx *ctx, const atp_plan_request *reqs, int n_req, void *
  *   cost_dev  float [K]: J of each candidate (as atp_plan computes it)
  *   grad_dev  float [H][K][2]: dJ/d(steering rate), dJ/d(acceleration);
  *             zero for a steering rate beyond its limit (the clamp)
- *   ckpt      control steps between stored states (0 selects 10).  A call keeps
- *             every Euler step's start state, 64 bytes per candidate and step,
- *             while that is at most 1 GiB; beyond, it recomputes segments of
- *             as many control steps as fit in it, at least ckpt, from stored
- *             states of 80 bytes per candidate and segment.  The results are
- *             the same bits either way and for every ckpt.
+ *   ckpt      bounds the call's device memory (0 selects 10).  Above 128 MiB it
+ *             takes at most (H / ckpt + b ckpt n_sub) x 320 bytes per
+ *             candidate, H / ckpt rounded up, with b = 2 while that is at most
+ *             16 GiB for all candidates and b = 1 (or 16 GiB) beyond.  Every
+ *             Euler step's start state (64 bytes per candidate and step) is
+ *             kept where that bound or 128 MiB holds them all; else the reverse
+ *             pass recomputes them in segments of as many control steps as fit
+ *             (at least ckpt), from one stored state of 80 bytes per candidate
+ *             and segment.  The results are the same bits either way and for
+ *             every ckpt.
  * K <= 2^28; F32X4 terrain only. */
 int atp_grad(atp_ctx *ctx, const atp_vehicle *veh, const atp_cost *cost, const atp_terrain *terrain,
              const atp_state *x0, const float *x0_dev, const float *ctrl_dev, int K, int H, float dt,

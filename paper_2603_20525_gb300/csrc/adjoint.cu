@@ -31,6 +31,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "adjoint.cuh"
 #include "duo.cuh"
 
@@ -559,22 +561,41 @@ cudaError_t launch_back(const BackParams &b, cudaStream_t stream)
     return cudaGetLastError();
 }
 
+// Bytes of one candidate: a record of the trace, a checkpoint, the adjoint
+// between segments, and what the forward pass leaves of its end.
+constexpr size_t kRecBytes = 64, kCkptBytes = 20 * sizeof(float), kLamBytes = 16 * sizeof(float),
+                 kEndBytes = sizeof(float4) + 2 * sizeof(int);
+// What `ckpt` bounds the workspace by, in bytes per candidate: a state in each
+// of four lanes, times the control steps' checkpoints and two segments' Euler
+// steps (one where two would take more than kTwoBytes).
+constexpr size_t kStateBytes = 4 * 20 * sizeof(float);
+
 }  // namespace
 
 GradPlan grad_plan(int K, int H, int n_sub, int ckpt)
 {
     const auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t per_step = (size_t)n_sub * kRecBytes;      // of one candidate's trace, per control step
+    const auto segments = [&](size_t seg) { return (H + seg - 1) / seg; };
+    const auto bytes = [&](size_t seg) {
+        const size_t n = segments(seg);
+        return seg * per_step + kEndBytes + (n > 1 ? n * kCkptBytes + kLamBytes : 0);
+    };
+    // what `ckpt` allows, and the most control steps that fit it: ckpt do
+    const auto allowed = [&](int b) { return kStateBytes * (segments(ckpt) + (size_t)b * ckpt * n_sub); };
+    const size_t bound = std::max(allowed(1), std::min(allowed(2), kTwoBytes / K));
+    size_t seg = std::min(std::max(bound / per_step, (size_t)ckpt), (size_t)H);
+    while (seg > (size_t)ckpt && bytes(seg) > bound) --seg;
+    if (H * per_step <= kWholeBytes / K) seg = H;
     GradPlan g;
-    const size_t per_step = (size_t)K * n_sub * 64;                     // bytes of trace per control step
-    const size_t fit = kTraceBytes / per_step;
-    g.seg = fit >= (size_t)H ? H : (int)(fit > (size_t)ckpt ? fit : (size_t)ckpt);
-    if (g.seg > H) g.seg = H;
-    g.n_seg = (H + g.seg - 1) / g.seg;
+    g.n_seg = (int)segments(seg);
+    g.seg = (int)segments(g.n_seg);                         // of one length, but for the last
+    g.n_seg = (int)segments(g.seg);
     size_t o = 0;
-    g.rec = o;  o = up(o + per_step * g.seg);
-    g.ckpt = o; o = up(o + (g.n_seg > 1 ? (size_t)g.n_seg * 20 * K * sizeof(float) : 0));
+    g.rec = o;  o = up(o + per_step * g.seg * K);
+    g.ckpt = o; o = up(o + (g.n_seg > 1 ? (size_t)g.n_seg * K * kCkptBytes : 0));
     g.fin = o;  o = up(o + (size_t)K * sizeof(float4));
-    g.lam = o;  o = up(o + (g.n_seg > 1 ? (size_t)K * 16 * sizeof(float) : 0));
+    g.lam = o;  o = up(o + (g.n_seg > 1 ? (size_t)K * kLamBytes : 0));
     g.ints = o; o = up(o + (size_t)K * 2 * sizeof(int));
     g.total = o;
     return g;

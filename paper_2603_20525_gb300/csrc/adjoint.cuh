@@ -11,10 +11,14 @@ struct PlanParams;
 // what the adjoint differentiates
 constexpr int kGradCost = 0, kGradMargin = 1;
 
-// Device memory of one adjoint call.  A trace (one record of 64 bytes per
-// candidate and Euler step) of up to kTraceBytes is kept whole; a longer one
-// is recomputed in segments of `seg` control steps from checkpoints.
-constexpr size_t kTraceBytes = (size_t)1 << 30;
+// Device memory of one adjoint call.  The trace (one record of 64 bytes per
+// candidate and Euler step) is kept whole up to kWholeBytes (the L2), and
+// beyond where the workspace that `ckpt` allows holds it (atp_grad in atp.h).
+// Else it is recomputed in segments of `seg` control steps from checkpoints,
+// and all but the last segment's share of the forward pass runs twice: 16384
+// candidates of 400 steps take 1.85 ms with a whole trace and 2.05 ms in two
+// segments, 65536 take 7.3 and 7.8 ms.
+constexpr size_t kWholeBytes = (size_t)128 << 20, kTwoBytes = (size_t)16 << 30;
 struct GradPlan {
     int seg, n_seg;                       // control steps per segment, segments
     size_t rec, ckpt, fin, lam, ints, total;   // byte offsets and size

@@ -76,8 +76,7 @@ enum {
 enum {
     ATP_OPT_COST_FP64 = 1,    /* accumulate the running cost in FP64 (default 0: FP32) */
     ATP_OPT_LANES = 2,        /* threads per candidate in atp_plan / atp_rollout: 0 chooses
-                                 by batch size (default), 1, 2 or 4 (eight in a small
-                                 plan) forces it */
+                                 by batch size (default), 1, 2 or 4 forces it */
     ATP_OPT_STAGE_TERRAIN = 3 /* side in nodes (2..120) of a texel window staged in shared
                                  memory by atp_plan / atp_rollout; 0 (default) off */
 };
@@ -176,9 +175,10 @@ size_t atp_terrain_bytes(int nx, int ny, int format);
  * in FP64 instead of FP32; ATP_OPT_LANES (0, 1, 2 or 4) sets the threads per
  * candidate of atp_plan and atp_rollout (one: more throughput once a batch
  * fills the GPU; two and four, in two warps that share the candidates' Euler
- * steps: lower latency for smaller batches; four means eight in plans of up to
- * 4864 candidates).  Every layout gives the same bits: all form the axle sums
- * and the force and moment totals in one order.
+ * steps: lower latency for smaller batches).  0, the default, chooses by batch
+ * size, eight threads among them up to 4864 candidates.  Every layout gives the
+ * same bits: all form the axle sums and the force and moment totals in one
+ * order.
  * ATP_OPT_STAGE_TERRAIN (0, or a side W from 2 to 120 nodes) stages a window
  * of the texels in shared memory (Sec. IV-D's cached terrain lookups): each
  * CTA of 512 threads first copies min(W, nx) x min(W, ny) texels (16 B each,
@@ -194,8 +194,9 @@ int atp_set_option(atp_ctx *ctx, int option, int value);
 
 /* Threads per candidate (1, 2 or 4) that atp_plan and atp_rollout on this
  * context use for a plan of N candidates: the ATP_OPT_LANES value if set,
- * else the library's choice by batch size.  Returns ATP_ERR_INVALID for a
- * NULL context or N < 1. */
+ * else the library's choice by batch size, where 4 stands for four or eight
+ * (up to 4864 candidates).  Returns ATP_ERR_INVALID for a NULL context or
+ * N < 1. */
 int atp_plan_lanes(const atp_ctx *ctx, int N);
 
 /* Build the texels of a terrain: per node the height, its slope f_x, f_y by

@@ -242,7 +242,8 @@ class Context:
         self._check(self.lib.atp_set_option(self.h, int(option), int(value)), "atp_set_option")
 
     def plan_lanes(self, N: int) -> int:
-        """Threads per candidate a plan of N candidates runs with."""
+        """Threads per candidate a plan of N candidates runs with: 1, 2 or 4,
+        the last also where the default takes eight (up to 4864)."""
         rc = self.lib.atp_plan_lanes(self.h, int(N))
         self._check(rc if rc < 0 else ATP_OK, "atp_plan_lanes")
         return rc

@@ -70,20 +70,21 @@ constexpr int kDuo4MaxN = 4864;
 constexpr int kDuo2MaxN = 16384;
 constexpr int kDuo1MaxN = 29184;
 
-// the layout of a plan of N candidates: `forced` (1, 2 or 4 threads, four
-// meaning eight where a plan of its size runs eight) if set, else by batch size
+// the layout of a plan of N candidates: `forced` (1, 2 or 4 threads per
+// candidate) if set, else by batch size
 inline int plan_layout(int forced, int N)
 {
-    const int four = N <= kDuo4MaxN ? kLayoutDuo4 : kLayoutDuo2;
-    if (forced) return forced == 4 ? four : forced;
-    return N <= kDuo2MaxN ? four : N <= kDuo1MaxN ? kLayoutDuo1 : kLayoutOne;
+    static_assert(kLayoutOne == 1 && kLayoutDuo1 == 2 && kLayoutDuo2 == 4, "a layout is its threads");
+    if (forced) return forced;
+    return N <= kDuo4MaxN ? kLayoutDuo4 : N <= kDuo2MaxN ? kLayoutDuo2 : N <= kDuo1MaxN ? kLayoutDuo1 : kLayoutOne;
 }
 inline int layout_candidates(int layout) { return kPlanBlock / layout; }       // per CTA
 inline long long layout_ctas(int layout, long long N)
 {
     return (N + layout_candidates(layout) - 1) / layout_candidates(layout);
 }
-// threads per candidate as ATP_OPT_LANES counts them: 1, 2 or 4 (or more)
+// threads per candidate as atp_plan_lanes counts them: 1, 2 or 4, where 4 may
+// be eight
 inline int plan_lanes(int forced, int N)
 {
     const int l = plan_layout(forced, N);

@@ -353,7 +353,8 @@ int atp_sample(atp_ctx *ctx, const float *prev_best_dev, int H_prev, int shift, 
 
 /* Diagnostic: evaluates the library's own FP32 elementary functions next to
  * CUDA's on n input pairs (a_i, b_i), writing 14 floats per pair to out_dev:
- * [sin a, cos a] (library), [sinf a, cosf a] (CUDA), atan2(a, b) (library),
+ * [sin a, cos a] (library; NaN where its forms with and without branches have
+ * not the same bits), [sinf a, cosf a] (CUDA), atan2(a, b) (library),
  * atan2f(a, b) (CUDA), 1/b (library reciprocal), 1.0f/b (IEEE division),
  * 1/sqrt(b) (library), rsqrtf(b) (CUDA), then a b + b by the packed
  * two-wide FMA and by the scalar one, and b - a by the packed two-wide

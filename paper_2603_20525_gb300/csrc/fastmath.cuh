@@ -78,9 +78,10 @@ __device__ __forceinline__ void sincos_r(float x, float &s, float &c)
 
 // sincos_r without the branch around the reduction: for |x| <= pi/4 the
 // quadrant is 0 and the reduction returns x itself, so the bits are
-// sincos_r's.  The quadrant comes from the low mantissa bits of a sum with
-// 1.5 x 2^23, not from a conversion.  SLOW = false leaves out CUDA's sincosf
-// for |x| >= kSincosMax: the caller tests for it and repeats with SLOW.
+// sincos_r's (atp_math_check compares them).  The quadrant comes from the low
+// mantissa bits of a sum with 1.5 x 2^23, not from a conversion.  SLOW = false
+// leaves out CUDA's sincosf for |x| >= kSincosMax: the caller tests for it and
+// repeats with SLOW.
 constexpr float kSincosMax = 131072.f;
 template <bool SLOW>
 __device__ __forceinline__ void sincos_g(float x, float &s, float &c)
@@ -98,6 +99,7 @@ __device__ __forceinline__ void sincos_g(float x, float &s, float &c)
     c = __uint_as_float(__float_as_uint(odd ? sr : cr) ^ (((q + 1u) & 2u) << 30));
     if (SLOW && fabsf(x) >= kSincosMax) sincosf(x, &s, &c);
 }
+
 // atan(r) for r in [0, 1] as r P(r^2), P of degree 8 fitted for minimum
 // maximum relative error (fit_atan.py): 1.1e-7 including FP32 evaluation.
 __device__ __forceinline__ float atan01(float r)

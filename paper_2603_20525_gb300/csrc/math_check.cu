@@ -1,11 +1,20 @@
 // math_check.cu - evaluates the rollout's own elementary functions
 // (fastmath.cuh) next to CUDA's library functions on the same inputs, so that
-// their error can be bounded on the GPU itself, and the packed two-wide FP32
-// operations next to their scalar forms.
+// their error can be bounded on the GPU itself, the two forms of sin and cos
+// against each other, and the packed two-wide FP32 operations next to their
+// scalar forms.
+#include <math_constants.h>
+
 #include "atp.h"
 #include "fastmath.cuh"
 
 namespace atp {
+
+// the same bits, or both NaN
+__device__ __forceinline__ bool same(float a, float b)
+{
+    return __float_as_uint(a) == __float_as_uint(b) || (a != a && b != b);
+}
 
 __global__ void math_check_kernel(const float *__restrict__ a, const float *__restrict__ b, int n,
                                   float *__restrict__ out)
@@ -16,6 +25,16 @@ __global__ void math_check_kernel(const float *__restrict__ a, const float *__re
     float s, c, s_ref, c_ref;
     sincos_r(x, s, c);
     sincosf(x, &s_ref, &c_ref);
+    // the rollouts' form without branches has sincos_r's bits: with the slow
+    // part for every argument, without it below kSincosMax.  NaN where not.
+    float sg, cg;
+    sincos_g<true>(x, sg, cg);
+    bool ok = same(s, sg) && same(c, cg);
+    if (!(fabsf(x) >= kSincosMax)) {
+        sincos_g<false>(x, sg, cg);
+        ok = ok && same(s, sg) && same(c, cg);
+    }
+    if (!ok) s = c = CUDART_NAN_F;
     float *o = out + (size_t)14 * i;
     o[0] = s;
     o[1] = c;

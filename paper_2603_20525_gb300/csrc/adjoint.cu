@@ -191,7 +191,7 @@ struct BackParams {
     Cost C;
     Terrain T;
     const float2 *ctrl;       // [H][K]
-    int K, H, n_sub;
+    int K, n_sub;
     float h;
     int objective;
     int k0, k1;               // this segment's control steps
@@ -226,16 +226,8 @@ __device__ __forceinline__ void linearise(const BackParams &p, int j, int e, flo
     sincos_r(ph, A.sph, A.cph);
     sincos_r(d, sd, cd);
     const float sth = A.sth, cth = A.cth, sph = A.sph, cph = A.cph;
-    float *R = A.R;
-    R[0] = A.cps * cth;
-    R[1] = fmaf(A.cps * sph, sth, -cph * A.sps);
-    R[2] = fmaf(cph * A.cps, sth, sph * A.sps);
-    R[3] = cth * A.sps;
-    R[4] = fmaf(sph * A.sps, sth, cph * A.cps);
-    R[5] = fmaf(cph * A.sps, sth, -A.cps * sph);
-    R[6] = -sth;
-    R[7] = cth * sph;
-    R[8] = cph * cth;
+    const float *R = A.R;
+    rotation(A.sps, A.cps, sth, cth, sph, cph, A.R);
     const Cell cx = cell_of<false>(s0.x, s0.y, T.inv_cell, T.nx), cy = cell_of<false>(s0.z, s0.w, T.inv_cell, T.ny);
     const unsigned base = texel_base(cx, cy, T.nx);
 
@@ -617,7 +609,6 @@ cudaError_t launch_grad(const PlanParams &p, const GradPlan &g, int objective, c
     b.T = p.T;
     b.ctrl = p.ctrl;
     b.K = p.N;
-    b.H = p.H;
     b.n_sub = p.n_sub;
     b.h = p.h;
     b.objective = objective;

@@ -686,7 +686,7 @@ extern "C" int atp_plan_est(atp_ctx *ctx, const atp_vehicle *veh, const atp_cost
     p.best_margin = best_margin_dev;
     p.scratch = (atp::Scratch *)ctx->scratch;
     p.acc64 = ctx->acc64;
-    cudaError_t e = atp::launch_est(p, true, (cudaStream_t)stream);
+    cudaError_t e = atp::launch_est(p, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "planar plan launch");
     return ATP_OK;
 }

@@ -410,7 +410,7 @@ __device__ __forceinline__ void est_forces(const PlanParams &p, EstDuo &sh, int 
     }
 }
 
-template <bool PER_X0, bool REDUCE, int TEX>
+template <bool PER_X0, int TEX>
 __global__ void __launch_bounds__(kPlanBlock) est_duo_kernel(const __grid_constant__ PlanParams p)
 {
     __shared__ EstDuo sh;
@@ -421,7 +421,6 @@ __global__ void __launch_bounds__(kPlanBlock) est_duo_kernel(const __grid_consta
     const bool geo = geometry_role(sh.flip);
     if (geo) est_geometry<PER_X0, TEX>(p, sh, j, c, live);
     else est_forces<PER_X0>(p, sh, j, c, live, J, margin, feasible);
-    if (!REDUCE) return;
     plan_tail(p, j, live && !geo, J, feasible, gridDim.x);
 }
 
@@ -431,7 +430,7 @@ __global__ void __launch_bounds__(kPlanBlock) est_duo_kernel(const __grid_consta
 // 181 / 178 at 65536; with a costmap 170 / 243 at 16384, 243 / 254 at 49152).
 constexpr int kEstDuoMaxN = 48640;
 
-template <bool PER_X0, bool REDUCE, int TEX>
+template <bool PER_X0, int TEX>
 __global__ void __launch_bounds__(kPlanBlock) est_kernel(const __grid_constant__ PlanParams p)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -439,42 +438,30 @@ __global__ void __launch_bounds__(kPlanBlock) est_kernel(const __grid_constant__
     float J = 0.f, margin = CUDART_INF_F;
     bool feasible = false;
     if (live) est_one<PER_X0, TEX>(p, j, J, margin, feasible);
-    if (!REDUCE) return;
     plan_tail(p, j, live, J, feasible, gridDim.x);
 }
 
 template <int TEX>
-cudaError_t launch_tex(const PlanParams &p, bool reduce, cudaStream_t stream)
+cudaError_t launch_tex(const PlanParams &p, cudaStream_t stream)
 {
     const bool per = p.x0_soa != nullptr;
     if (p.N <= kEstDuoMaxN) {
         const dim3 grid((unsigned)((p.N + 31) / 32));
-        if (reduce) {
-            if (per) est_duo_kernel<true, true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-            else est_duo_kernel<false, true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-        } else {
-            if (per) est_duo_kernel<true, false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-            else est_duo_kernel<false, false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-        }
-        return cudaGetLastError();
-    }
-    const dim3 grid((unsigned)(((size_t)p.N + kPlanBlock - 1) / kPlanBlock));
-    if (reduce) {
-        if (per) est_kernel<true, true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-        else est_kernel<false, true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
+        if (per) est_duo_kernel<true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
+        else est_duo_kernel<false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
     } else {
-        if (per) est_kernel<true, false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
-        else est_kernel<false, false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
+        const dim3 grid((unsigned)(((size_t)p.N + kPlanBlock - 1) / kPlanBlock));
+        if (per) est_kernel<true, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
+        else est_kernel<false, TEX><<<grid, kPlanBlock, 0, stream>>>(p);
     }
     return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_est(const PlanParams &p, bool reduce, cudaStream_t stream)
+cudaError_t launch_est(const PlanParams &p, cudaStream_t stream)
 {
-    return p.tex_format == TEX_F32 ? launch_tex<TEX_F32>(p, reduce, stream)
-                                   : launch_tex<TEX_BF16>(p, reduce, stream);
+    return p.tex_format == TEX_F32 ? launch_tex<TEX_F32>(p, stream) : launch_tex<TEX_BF16>(p, stream);
 }
 
 }  // namespace atp

@@ -9,6 +9,6 @@
 
 namespace atp {
 
-cudaError_t launch_est(const PlanParams &p, bool reduce, cudaStream_t stream);
+cudaError_t launch_est(const PlanParams &p, cudaStream_t stream);
 
 }  // namespace atp

@@ -421,7 +421,7 @@ def run_variants(ctx, dev, stream, flush, steps=10):
                steps, 3, stream, flush)
     out["plain_plan"] = {"workload": f"plain: {wp.N} candidates x H={wp.H} at dt={wp.dt} s "
                                      f"({wp.n_sub} Euler steps), 256^2 map at 0.2 m, "
-                                     f"{ctx.plan_lanes(wp.N)} threads per candidate",
+                                     f"{ctx.plan_lanes(wp.N)} threads per candidate (4: eight up to 4864)",
                          "ms_per_plan": ms, "rollout_steps_per_s": wp.N * wp.H / (ms / 1e3)}
     t = gen.terrain_tile(2048, 5, lod_sigma=0.0)
     h = torch.as_tensor(t.heights).to(dev)
@@ -661,7 +661,8 @@ def main():
                            "p99": float(np.percentile(per_step, 99))},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": recorded_traffic(args.workload),
-                         "kernel": "plan_duo_kernel (fused rollout + argmin)",
+                         "kernel": ("plan_kernel" if ctx.plan_lanes(w.N) == 1 else "plan_duo_kernel") +
+                                   " (fused rollout + argmin)",
                          "note": f"{flops} algorithmic FP32 flops per Euler step (counted by the "
                                  f"oracle's counting scalar) x {substeps} Euler steps per launch; "
                                  f"peak = {sms} SMs (device query) x {FP32_LANES_PER_SM} FP32 lanes x 2 "

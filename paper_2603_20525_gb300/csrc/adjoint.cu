@@ -13,13 +13,15 @@
 // linearises one Euler step (the 13 x 13 matrix by which the step's adjoint
 // changes, column by column into shared memory), and then one warp runs the
 // recursion lam <- lam + M lam + c over those steps, one column per lane.
-// The recursion's step is 13 shuffles and 13 FMAs, instead of the step's
-// whole forward and reverse arithmetic on the serial chain.  Walking the
-// steps back with their arithmetic on the chain, beside a recomputation from
-// checkpoints, took 716 us for 64 candidates of 400 steps, 753 us for 4096 of
-// 300 and 597 us for 8000 of 200; this way they take 208, 420 and 500 us.  The
-// forward chain bounds the first (about 150 us), the linearisation's issue and
-// the seven warps per SM that its shared memory holds the others.
+// The recursion's step is one round trip through shared memory and 13 FMAs,
+// instead of the step's whole forward and reverse arithmetic on the serial
+// chain.  Walking the steps back with their arithmetic on the chain, beside a
+// recomputation from checkpoints, took (ms) 0.73 for 64 candidates of 400
+// steps, 0.78 for 4096 of 300, 1.28 and 2.62 for 16384 of 200 and 400, 4.16 for
+// 32768 of 400 and 7.46 for 131072 of 200; this way they take 0.21, 0.43, 0.95,
+// 1.85, 3.86 and 6.91.  The forward chain bounds the first (about 0.15), the
+// linearisation's issue and the seven warps per SM that its shared memory holds
+// the others.
 //
 // Linearising a step differentiates the Euler update, the state derivative
 // A(xi) + B zeta, the force and moment sums, every wheel (contact kinematics,

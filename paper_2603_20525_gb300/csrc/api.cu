@@ -325,8 +325,9 @@ cudaError_t launch_plan_for(const atp_ctx *ctx, atp::PlanParams &p, const atp_te
 // the waves of a plan that alone overfills the 912 CTAs resident on 152 SMs),
 // and at least the SMs' time for all its candidates; a layout of more threads
 // shortens the first and costs more of the second.  The layout with the
-// smallest cube root of the two bounds' cubes wins: within 10 % of the measured
-// time on ten serving batches of 1024 to 93184 candidates.  One layout for the
+// smallest cube root of the two bounds' cubes wins: on eleven batches of 1024 to
+// 124928 candidates in one to eight plans it is the fastest of the four but for
+// one (1510 us on one thread, 1493 on two).  One layout for the
 // whole batch: mixes of layouts were measured slower than either alone (seven
 // plans of 4096: 1.07 ms mixed, 0.74 ms on two threads, 0.91 ms on one; the
 // SMs then alternate between the layouts' loops).  The CTAs go in the order
@@ -334,7 +335,9 @@ cudaError_t launch_plan_for(const atp_ctx *ctx, atp::PlanParams &p, const atp_te
 int choose_layout(const atp_plan_request *q, const int *ns, int n)
 {
     // cycles per Euler step with the GPU nearly idle, and SM cycles per
-    // candidate and Euler step with it full, from a sweep on a GB300
+    // candidate and Euler step with it full, from sweeps on a GB300 (one
+    // thread's first is from before its four sincos lost their branches: 1480
+    // cycles now)
     constexpr int kL[4] = {atp::kLayoutOne, atp::kLayoutDuo1, atp::kLayoutDuo2, atp::kLayoutDuo4};
     constexpr double kLatency[4] = {1744., 1200., 1000., 810.}, kBusy[4] = {9.0, 10.3, 12.9, 26.};
     constexpr double kSms = 152., kWave = 6 * kSms;

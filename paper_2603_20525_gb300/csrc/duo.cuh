@@ -599,7 +599,7 @@ __device__ __forceinline__ void duo_forces(const PlanParams &p, const Tr &tr, Du
 }
 
 // Whether this warp is its pair's geometry warp.  Warps w and w + 4 share an
-// SM sub-partition, and the geometry warp issues about 1.6 times the forces
+// SM sub-partition, and the geometry warp issues about 1.3 times the forces
 // warp's instructions: the roles alternate by the CTA's warp slots, so that
 // the sub-partitions get both kinds (the scaled plan 407 -> 336 us with two
 // lanes).  The shuffle makes the answer uniform over the warp, so that the

@@ -51,21 +51,25 @@ constexpr int kPlanBlock = 64;
 // thread, or two warps that share 32, 16 or 8 candidates (one, two or four
 // lanes of each warp per candidate).  All give the same bits.
 constexpr int kLayoutOne = 1, kLayoutDuo1 = 2, kLayoutDuo2 = 4, kLayoutDuo4 = 8;
-// The lines lie where the next layout becomes the faster one (ms per plan on a
-// GB300, scaled workload, H = 100, 4 Euler steps per control step):
+// ms per plan on a GB300, scaled workload, H = 100, 4 Euler steps per control
+// step, terrain seed 5:
 //   candidates        8 threads   4 threads   2 threads   1 thread
-//   1024                0.160       0.193       0.243       0.330
-//   4096                0.177       0.194       0.248       0.339
-//   8192                0.241       0.216       0.248       0.337
-//   12288               0.385       0.266       0.281       0.344
-//   16384               0.420       0.315       0.296       0.344
-//   20480               0.592       0.473       0.369       0.424
-//   28672                           0.505       0.383       0.430
-//   32768                           0.565       0.615       0.436
+//   1024                0.158       0.180       0.225       0.287
+//   4096                0.176       0.182       0.232       0.297
+//   4864                0.178       0.182       0.227       0.295
+//   8192                0.242       0.216       0.231       0.299
+//   12288               0.390       0.259       0.270       0.304
+//   16384               0.424       0.315       0.284       0.305
+//   20480               0.601       0.471       0.355       0.401
+//   28672               0.698       0.508       0.371       0.410
+//   32768               0.828       0.565       0.610       0.415
 // 4864 = 152 x 4 x 8 candidates is four CTAs per SM on eight threads and 29184
-// = 152 x 6 x 32 the one wave of six CTAs per SM on two; between four and two
-// threads the order at 16384 depends on the terrain (0.296 to 0.376 ms on two,
-// 0.315 to 0.349 ms on four over five seeds).
+// = 152 x 6 x 32 the one wave of six CTAs per SM on two; there the next layout
+// becomes the faster one.  Four threads and two cross between 14336 candidates
+// (means of five terrains each of three workloads, four against two: 0.279 /
+// 0.303, 0.277 / 0.308 and 0.259 / 0.269 ms) and 16384 (0.327 / 0.314, 0.326 /
+// 0.319, 0.309 / 0.277): up to 10 % is lost just below the line, where one
+// workload's terrains spread more than that (0.285 to 0.369 ms on two).
 constexpr int kDuo4MaxN = 4864;
 constexpr int kDuo2MaxN = 16384;
 constexpr int kDuo1MaxN = 29184;
